@@ -21,8 +21,8 @@
 //  * 1/r is one MUFU rsqrt.approx per pair;
 //  * each target keeps an FP32 partial per staged tile, folded into an (hi, lo) two-sum pair;
 //  * surface points apply the dipole layer in its dy -> 0 limit sharing the monopole's rsqrt.
-// FP64 path: the same structure in double precision with the central-difference dipole in
-// the cancellation-free form 2 (R_tau - x.yhat) / (d+ d- (d+ + d-)).
+// FP64 path: the same items in double precision with the central-difference dipole in the
+// cancellation-free form 2 (R_tau - x.yhat) / (d+ d- (d+ + d-)).
 #include <math.h>
 
 #include "df64.cuh"
@@ -136,8 +136,35 @@ void launch_pairs_f32(int cfg, int grid, const SysDev* sys, PairWork w1, PairWor
 }
 
 // ---------------------------------------------------------------------------------------
-// FP64 comparator path: one target per thread, plain staged loads.
+// FP64 path: one target per thread, plain staged loads.  Bound by the FP64 pipe (1.6 FMA per
+// clock and SM, 1/73 of FP32), so the kernel counts FP64 operations: 12 a pair and 33 a surface
+// point.
+//  * 1/r is the MUFU start value and one third-order step (5 operations), not a square root and
+//    a division (about 20).
+//  * Surface points: with d0 = |x - y|, h = dy/2 and B = R_tau - x.yhat, the two shells of the
+//    dipole are at d_-+^2 = d0^2 + h^2 -+ 2 h B = A -+ C, so that
+//      2 B / (d_+ d_- (d_+ + d_-)) = 2 B / (s sqrt(2 A + 2 s)),  s = d_+ d_- = sqrt(A^2 - C^2)
+//    (two reciprocal roots, no division), and B = (R_tau^2 - |x|^2 + d0^2) / (2 R_tau), every term
+//    positive inside the cavity, needs no unit vector of the point.  A, B and C are taken in units
+//    of R_tau, so that A^2 stays in range for a cavity of any size.
+// A step of N = 1999, M = 1000, p = 20 (one GB300): 1300 us with the square roots and divisions of
+// the plain definition (five roots and divisions and a unit vector per surface point), 500 us so,
+// at the same error against the 64-bit definition (1.2e-15).
 constexpr int kF64Threads = kF64TargetsPerBlock;
+
+// 1/sqrt(x): the approximate reciprocal root (relative error below 2^-19), then, with e = 1 - x y^2,
+// y + y e (1/2 + 3/8 e) (the next term, 5/16 e^3, is below 2^-56).  Arguments whose exponent leaves
+// no room for the step (zero, subnormal, near overflow, not finite) take the square root and the
+// division.
+__device__ __forceinline__ double rsqrt_f64(double x)
+{
+  const unsigned int top = (unsigned int)__double2hiint(x) >> 20;  // sign and exponent
+  if (top - 0x040u > 0x780u - 0x040u) return 1.0 / sqrt(x);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
 
 __global__ __launch_bounds__(kF64Threads) void k_pairs_f64(const SysDev* __restrict__ sys, PairWork w1,
                                                            PairWork w2, const dbl4* __restrict__ src64,
@@ -166,45 +193,43 @@ __global__ __launch_bounds__(kF64Threads) void k_pairs_f64(const SysDev* __restr
     const int i = it.y * kF64Threads + tid;
     const dbl4 tg = src64[S.src + (i < n ? i : it.y * kF64Threads)];
     const ChunkInfo ch = decode_chunk(S, it.z);
-    const double Rt = S.Rtau, rm = S.Rtau - 0.5 * S.dy, rp = S.Rtau + 0.5 * S.dy;
+    // surface points, in units of R_tau: 1/R_tau^2, dy, (dy/2)^2 and (1 - |x|^2)/2
+    const double iR2 = S.inv_Rt * S.inv_Rt, dy = S.dy * S.inv_Rt, h2 = 0.25 * dy * dy;
+    const double bx = 0.5 - 0.5 * (tg.x * tg.x + tg.y * tg.y + tg.z * tg.z) * iR2, hR2 = 0.5 * iR2;
     double acc = 0.0;
     for (int t0 = 0; t0 < ch.count; t0 += kF64Threads) {
       const int cnt = min(kF64Threads, ch.count - t0);
       if (tid < cnt) {
         if (ch.type == 2) {
           shA[tid] = surf64_a[ch.off + t0 + tid];
-          shB[tid] = surf64_b[ch.off + t0 + tid];
+          shB[tid] = 2.0 * surf64_b[ch.off + t0 + tid] * S.inv_Rt * S.inv_Rt;
         } else {
           shA[tid] = src64[ch.off + t0 + tid];
         }
       }
       __syncthreads();
       if (ch.type == 2) {
+#pragma unroll 2
         for (int s = 0; s < cnt; ++s) {
           const dbl4 y = shA[s];
-          const double D = shB[s];
-          const double dx = tg.x - y.x, dy = tg.y - y.y, dz = tg.z - y.z;
-          acc += y.w * rsqrt(dx * dx + dy * dy + dz * dz);
-          const double rho = sqrt(y.x * y.x + y.y * y.y + y.z * y.z);
-          const double hx = y.x / rho, hy = y.y / rho, hz = y.z / rho;
-          const double mx = tg.x - rm * hx, my = tg.y - rm * hy, mz = tg.z - rm * hz;
-          const double px = tg.x - rp * hx, py = tg.y - rp * hy, pz = tg.z - rp * hz;
-          const double dm = sqrt(mx * mx + my * my + mz * mz);
-          const double dp = sqrt(px * px + py * py + pz * pz);
-          const double xy = tg.x * hx + tg.y * hy + tg.z * hz;
-          acc += D * 2.0 * (Rt - xy) / (dp * dm * (dp + dm));
+          const double dx = tg.x - y.x, dy_ = tg.y - y.y, dz = tg.z - y.z;
+          const double d2 = dx * dx + dy_ * dy_ + dz * dz;
+          acc = fma(y.w, rsqrt_f64(d2), acc);
+          const double B = fma(d2, hR2, bx), A = fma(d2, iR2, h2), C = dy * B;
+          const double m = fma(A, A, -(C * C));
+          const double rm = rsqrt_f64(m);
+          const double s2 = A + m * rm;  // (d_+ + d_-)^2 / 2
+          acc = fma(shB[s] * B, rm * rsqrt_f64(s2 + s2), acc);
         }
       } else {
-        const int sb = ch.first + t0;
+        // the charge itself, a real source: skipped
+        const int self = ch.type == 0 ? i - (ch.first + t0) : -1;
+#pragma unroll 4
         for (int s = 0; s < cnt; ++s) {
-          const dbl4 h = shA[s];
-          if (ch.type == 0 && sb + s == i) continue;
-          // separately rounded IEEE operations and a correctly rounded sqrt and division: the
-          // distance of a charge to its own nearby Kelvin image is ill-conditioned, so this path
-          // evaluates it exactly as the plain definition does
-          const double dx = tg.x - h.x, dy = tg.y - h.y, dz = tg.z - h.z;
-          const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-          acc += h.w / sqrt(r2);
+          const dbl4 r = shA[s];
+          const double dx = tg.x - r.x, dy_ = tg.y - r.y, dz = tg.z - r.z;
+          const double v = r.w * rsqrt_f64(dx * dx + dy_ * dy_ + dz * dz);
+          acc += s == self ? 0.0 : v;
         }
       }
       __syncthreads();
