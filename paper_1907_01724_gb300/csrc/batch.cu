@@ -76,7 +76,7 @@ int Engine::autotune(int reps, int* best_out, float* best_ms_out)
   reps = std::max(1, reps);
   const std::vector<int64_t> ns = cur_ns;
   size_t need = 0;
-  for (int c = 0; c < pair_config_count(); ++c) need = std::max(need, make_layout(ns, c).bytes);
+  for (int c = 0; c < pair_config_count(); ++c) need = std::max(need, make_layout(ns, c, true).bytes);
   if (need > ws_cap && ws_user) return fail(HSMA_E_OOM, "attached workspace too small to autotune");
   if (need > ws_cap) {
     // grow, keeping the inputs (at the same offsets in every layout)
@@ -247,7 +247,7 @@ int hsma_batch_workspace_size(hsma_batch_t* b, const int64_t* n, size_t* bytes)
   // serves the autotuner
   size_t mx = 0;
   const int ncfg = b->e->prec == HSMA_FP64 ? 1 : hsma::pair_config_count();
-  for (int c = 0; c < ncfg; ++c) mx = std::max(mx, b->e->make_layout(ns, c).bytes);
+  for (int c = 0; c < ncfg; ++c) mx = std::max(mx, b->e->make_layout(ns, c, true).bytes);
   *bytes = mx;
   return HSMA_OK;
 }

@@ -180,7 +180,96 @@ void Engine::drop_graphs()
 }
 
 // ---------------------------------------------------------------------------------------
-Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg) const
+// Whether an item is a real/Kelvin one.
+static bool is_rk(const Layout& L, const int4& it) { return it.z < L.sd[it.x].ncr + L.sd[it.x].nck; }
+
+// Items longest first (cost ~ targets x sources x per-source weight); among real/Kelvin items of
+// equal cost, the blocks nearest each other first: charges are in spatial order, so the block
+// distance |c - b| tracks their separation, and near blocks take the slower forms (more checked
+// boxes, their close pairs in the exact form; 1.5-2x the time of a far pair of blocks measured on
+// GB300), so the far, fast ones are left for the end of a launch.  Each item's key is formed once
+// (a comparison that evaluated both costs made the sort most of a layout: with it, and a sort in
+// every one of the layouts that a workspace size needs, the first pass of 512 cavities took 618
+// ms; 67 ms so).
+void Engine::sort_items(const Layout& L, std::vector<int4>& items, bool field) const
+{
+  const bool sym = prec != HSMA_FP64;
+  struct Keyed {
+    int64_t cost;
+    int gap, at;
+  };
+  std::vector<Keyed> keys(items.size());
+  for (size_t i = 0; i < items.size(); ++i) {
+    int4& it = items[i];
+    it.w = 0;
+    const SysDev& d = L.sd[it.x];
+    const bool rk = is_rk(L, it);
+    const int cb = it.z < d.ncr ? it.z : it.z - d.ncr;
+    int64_t nt, ns_, w = 10;
+    if (sym && !field && rk) {
+      // a real/Kelvin block against a chunk: both ways off the diagonal, one way on it (with
+      // the self box checked)
+      nt = std::min<int64_t>(d.chunk, d.n - (int64_t)it.y * d.chunk);
+      w = 12;
+    } else {
+      const int64_t tbk = field ? L.TBf : d.tb;
+      nt = std::min<int64_t>(tbk, d.n - (int64_t)it.y * tbk);
+    }
+    if (rk) {
+      ns_ = std::min<int64_t>(d.chunk, d.n - (int64_t)cb * d.chunk);
+    } else {
+      ns_ = std::min<int64_t>(d.chunk_s, d.M - (int64_t)(it.z - d.ncr - d.nck) * d.chunk_s);
+      w = 13;
+    }
+    keys[i] = Keyed{nt * ns_ * w, rk && !field ? std::abs(cb - it.y) : 0, (int)i};
+  }
+  std::sort(keys.begin(), keys.end(), [](const Keyed& x, const Keyed& y) {
+    if (x.cost != y.cost) return x.cost > y.cost;
+    return x.gap != y.gap ? x.gap < y.gap : x.at < y.at;
+  });
+  std::vector<int4> sorted(items.size());
+  for (size_t i = 0; i < items.size(); ++i) sorted[i] = items[keys[i].at];
+  items.swap(sorted);
+}
+
+// The real/Kelvin items to the front, in order; their number.
+int Engine::split_items(const Layout& L, std::vector<int4>& items) const
+{
+  return (int)(std::stable_partition(items.begin(), items.end(), [&](const int4& it) { return is_rk(L, it); }) -
+               items.begin());
+}
+
+// The item lists of the field pass: on the FP64 path those of the pair kernel, on the FP32 path
+// every (target block, chunk) one way; made and uploaded by the layout's first field pass.
+int Engine::make_field_items()
+{
+  if (L.field_items) return HSMA_OK;
+  if (prec == HSMA_FP64) {
+    L.it4f = L.it4;
+  } else {
+    L.it4f.clear();
+    L.it4f.reserve(L.n4f);
+    for (int s = 0; s < (int)L.sd.size() && !L.tree; ++s) {
+      const SysDev& d = L.sd[s];
+      const int nch = d.ncr + d.nck + d.ncs, ntb = (d.n + L.TBf - 1) / L.TBf;
+      for (int tb = 0; tb < ntb; ++tb)
+        for (int c = 0; c < nch; ++c) L.it4f.push_back(make_int4(s, tb, c, 0));
+    }
+  }
+  sort_items(L, L.it4f, true);
+  L.it4fx = L.it4f;
+  L.nRKf = split_items(L, L.it4fx);
+  if (!L.it4f.empty()) {
+    CK(cudaMemcpyAsync(it4f_d, L.it4f.data(), sizeof(int4) * L.it4f.size(), cudaMemcpyHostToDevice, stream));
+    CK(cudaMemcpyAsync(it4fx_d, L.it4fx.data(), sizeof(int4) * L.it4fx.size(), cudaMemcpyHostToDevice, stream));
+    CK(cudaStreamSynchronize(stream));
+  }
+  L.field_items = true;
+  return HSMA_OK;
+}
+
+// sizes_only: the workspace plan alone (the pair items are counted, not listed).
+Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_only) const
 {
   Layout L;
   const int nsys = (int)spec.size();
@@ -333,22 +422,25 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg) const
     for (int b = 0; b < d.sort_parts; ++b) L.itsort.push_back(make_int2(s, b));
     const int nch = d.ncr + d.nck + d.ncs;
     if (prec == HSMA_FP64) {
-      for (int tb = 0; tb < d.n_tb; ++tb)
+      L.n4 += (size_t)d.n_tb * nch;
+      for (int tb = 0; !sizes_only && tb < d.n_tb; ++tb)
         for (int c = 0; c < nch; ++c) L.it4.push_back(make_int4(s, tb, c, 0));
     } else if (n > 0) {
       // the pair kernel: each unordered pair of real/Kelvin blocks once (none with the tree),
       // surface items per group
-      for (int b = 0; b < (L.tree ? 0 : d.ncr); ++b)
-        for (int c = b; c < d.ncr; ++c) {
-          L.it4.push_back(make_int4(s, b, c, 0));
-          L.it4.push_back(make_int4(s, b, d.ncr + c, 0));
-        }
-      for (int tb = 0; tb < d.n_tb; ++tb)
-        for (int c = d.ncr + d.nck; c < nch; ++c) L.it4.push_back(make_int4(s, tb, c, 0));
-      // the field kernel: every (target block, chunk) one way (no field pass with the tree)
-      const int ntbf = L.tree ? 0 : (int)((n + TBf - 1) / TBf);
-      for (int tb = 0; tb < ntbf; ++tb)
-        for (int c = 0; c < nch; ++c) L.it4f.push_back(make_int4(s, tb, c, 0));
+      L.n4 += (L.tree ? 0 : (size_t)d.ncr * (d.ncr + 1)) + (size_t)d.n_tb * d.ncs;
+      if (!sizes_only) {
+        for (int b = 0; b < (L.tree ? 0 : d.ncr); ++b)
+          for (int c = b; c < d.ncr; ++c) {
+            L.it4.push_back(make_int4(s, b, c, 0));
+            L.it4.push_back(make_int4(s, b, d.ncr + c, 0));
+          }
+        for (int tb = 0; tb < d.n_tb; ++tb)
+          for (int c = d.ncr + d.nck; c < nch; ++c) L.it4.push_back(make_int4(s, tb, c, 0));
+      }
+      // the field kernel: every (target block, chunk) one way (no field pass with the tree); the
+      // list itself is made by the first field pass (make_field_items)
+      if (!L.tree) L.n4f += (size_t)((n + TBf - 1) / TBf) * nch;
     }
     chg += n;
     surf += sp.M;
@@ -398,56 +490,13 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg) const
         for (int b = 0; b < (spec[s].M + pts - 1) / pts; ++b) L.it3m.push_back(make_int2(s, b));
     }
   }
-  // longest pair items first (cost ~ targets x sources x per-source weight); among real/Kelvin
-  // items of equal cost, the blocks nearest each other first: charges are in spatial order, so
-  // the block distance |c - b| tracks their separation, and near blocks take the slower forms
-  // (more checked boxes, their close pairs in the exact form; 1.5-2x the time of a far pair of
-  // blocks measured on GB300), so the far, fast ones are left for the end of a launch
-  const bool sym = prec != HSMA_FP64;
-  auto cost_of = [&](const int4& it, bool field) {
-    const SysDev& d = L.sd[it.x];
-    const bool rk = it.z < d.ncr + d.nck;
-    const int cb = it.z < d.ncr ? it.z : it.z - d.ncr;
-    int64_t nt, ns_, w = 10;
-    if (sym && !field && rk) {
-      // a real/Kelvin block against a chunk: both ways off the diagonal, one way on it (with
-      // the self box checked)
-      nt = std::min<int64_t>(d.chunk, d.n - (int64_t)it.y * d.chunk);
-      w = 12;
-    } else {
-      const int64_t tbk = field ? TBf : d.tb;
-      nt = std::min<int64_t>(tbk, d.n - (int64_t)it.y * tbk);
-    }
-    if (rk) {
-      ns_ = std::min<int64_t>(d.chunk, d.n - (int64_t)cb * d.chunk);
-    } else {
-      ns_ = std::min<int64_t>(d.chunk_s, d.M - (int64_t)(it.z - d.ncr - d.nck) * d.chunk_s);
-      w = 13;
-    }
-    return nt * ns_ * w;
-  };
-  auto is_rk = [&](const int4& it) { return it.z < L.sd[it.x].ncr + L.sd[it.x].nck; };
-  for (auto& it : L.it4) it.w = 0;
-  auto gap_of = [&](const int4& it) {
-    const SysDev& d = L.sd[it.x];
-    if (it.z >= d.ncr + d.nck) return 0;
-    return std::abs((it.z < d.ncr ? it.z : it.z - d.ncr) - it.y);
-  };
-  std::stable_sort(L.it4.begin(), L.it4.end(), [&](const int4& x, const int4& y) {
-    const int64_t cx = cost_of(x, false), cy = cost_of(y, false);
-    return cx != cy ? cx > cy : gap_of(x) < gap_of(y);
-  });
+  L.TBf = TBf;
+  if (prec == HSMA_FP64) L.n4f = L.n4;
+  if (!sizes_only) sort_items(L, L.it4, false);
   // the overlapped pass launches the real/Kelvin items (which need only the records) apart from
   // the surface items (which wait for the coefficient chain)
   L.it4x = L.it4;
-  L.nRK = (int)(std::stable_partition(L.it4x.begin(), L.it4x.end(), is_rk) - L.it4x.begin());
-  // the field pass: on the FP64 path the same one-way list; on the FP32 path its own
-  if (!sym) L.it4f = L.it4;
-  for (auto& it : L.it4f) it.w = 0;
-  std::stable_sort(L.it4f.begin(), L.it4f.end(),
-                   [&](const int4& x, const int4& y) { return cost_of(x, true) > cost_of(y, true); });
-  L.it4fx = L.it4f;
-  L.nRKf = (int)(std::stable_partition(L.it4fx.begin(), L.it4fx.end(), is_rk) - L.it4fx.begin());
+  if (!sizes_only) L.nRK = split_items(L, L.it4x);
   {
     // a sort block's share: all of a one-block system, else twice the mean share of its blocks
     // (a denser run of cells spills to the scratch buffer)
@@ -466,7 +515,7 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg) const
   L.totBoxes = boxes;
   L.mom_stride = (int)align_up((size_t)L.maxP + 1, 2);
   L.nw = nw;
-  L.pair_grid = (int)std::max<size_t>(1, std::min<size_t>((L.it4.size() + nw - 1) / nw, (size_t)slots));
+  L.pair_grid = (int)std::max<size_t>(1, std::min<size_t>((L.n4 + nw - 1) / nw, (size_t)slots));
 
   // workspace plan
   size_t off = 0;
@@ -555,10 +604,10 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg) const
   L.o_it3 = take(sizeof(int2) * L.it3.size());
   L.o_it3m = take(sizeof(int2) * L.it3m.size());
   L.o_it5 = take(sizeof(int2) * L.it5.size());
-  L.o_it4 = take(sizeof(int4) * L.it4.size());
-  L.o_it4x = take(sizeof(int4) * L.it4x.size());
-  L.o_it4f = take(sizeof(int4) * L.it4f.size());
-  L.o_it4fx = take(sizeof(int4) * L.it4fx.size());
+  L.o_it4 = take(sizeof(int4) * L.n4);
+  L.o_it4x = take(sizeof(int4) * L.n4);
+  L.o_it4f = take(sizeof(int4) * L.n4f);
+  L.o_it4fx = take(sizeof(int4) * L.n4f);
   L.sel.resize(nsys);
   L.selrng.resize(nsys);
   for (int s = 0; s < nsys; ++s) {
@@ -737,10 +786,6 @@ int Engine::set_sizes(const std::vector<int64_t>& ns)
     CK(cudaMemcpyAsync(it4_d, L.it4.data(), sizeof(int4) * L.it4.size(), cudaMemcpyHostToDevice, stream));
   if (!L.it4x.empty())
     CK(cudaMemcpyAsync(it4x_d, L.it4x.data(), sizeof(int4) * L.it4x.size(), cudaMemcpyHostToDevice, stream));
-  if (!L.it4f.empty())
-    CK(cudaMemcpyAsync(it4f_d, L.it4f.data(), sizeof(int4) * L.it4f.size(), cudaMemcpyHostToDevice, stream));
-  if (!L.it4fx.empty())
-    CK(cudaMemcpyAsync(it4fx_d, L.it4fx.data(), sizeof(int4) * L.it4fx.size(), cudaMemcpyHostToDevice, stream));
   if (!L.itsb.empty())
     CK(cudaMemcpyAsync(itsb_d, L.itsb.data(), sizeof(int2) * L.itsb.size(), cudaMemcpyHostToDevice, stream));
   if (!L.itord.empty())
@@ -1373,6 +1418,8 @@ int Engine::field()
   CK(cudaSetDevice(device));
   int rc = ensure_field_buffers();
   if (rc) return rc;
+  rc = make_field_items();
+  if (rc) return rc;
   if (build_pending && overlap && !L.itord.empty()) {
     enter();
     rc = prepare_inputs();
@@ -1473,17 +1520,43 @@ int Engine::decode_status(int st)
   return HSMA_OK;
 }
 
+// The configuration with the given CTA size, targets per thread and items per worker slot.
+static int config_of(int threads, int k, int items_per_slot)
+{
+  for (int c = 0; c < pair_config_count(); ++c) {
+    const PairConfig p = pair_config(c);
+    if (p.threads == threads && p.k == k && p.items_per_slot == items_per_slot) return c;
+  }
+  return 0;
+}
+
 // Pair-sum tile configuration for a set of sizes: the autotuned choice if one is cached for
-// this size bucket, else a size heuristic.
+// this size bucket, else by the pair work W = sum N (2N + 1.3 M) of the engine: groups of 32 K
+// targets, small while there are fewer items than warps (a launch is then as long as its longest
+// item), large when items abound (a staged source then serves more targets).  Step times of one
+// cavity on a GB300, in us, for K = 1, 2 and 4 (128, 64 and 64 threads; 4, 4 and 8 items per slot):
+//   N = 700 (W = 1.9e6) 33.0, 35.6, 43.4; N = 2000 (1.1e7) 39.2, 41.5, 53.6;
+//   4 x 2000 (4.2e7) 59.5, 53.1, 58.5; N = 4999 (5.6e7) 66.5, 57.7, 61.8;
+//   N = 10000 (2.3e8) 154, 114, 107.6; 16 x 3000 (3.3e8) 270, 221, 205.5;
+//   N = 40000 (3.3e9) 1445, 903, 718.
+// (At N = 2000 the smallest groups would save 2 us a step, but their 63 x 64 items cost a first pass
+// 0.18 ms more.)
+// Larger CTAs hold their SM slots until their slowest warp is done: (128, 4) with 4 items per slot
+// takes 110.7, 258.8 and 735.5 at N = 10000, 20000 and 40000 against 107.6, 251.1 and 717.8.
 int Engine::choose_config(const std::vector<int64_t>& ns) const
 {
   if (forced_cfg >= 0) return forced_cfg;
   int64_t tot = 0;
-  for (auto v : ns) tot += v;
+  double W = 0.0;
+  for (size_t s = 0; s < ns.size(); ++s) {
+    tot += ns[s];
+    W += (double)ns[s] * (2.0 * (double)ns[s] + 1.3 * spec[s].M);
+  }
   const int bucket = tune_bucket(tot, (int)ns.size());
   for (const auto& e : tuned)
     if (e.bucket == bucket) return e.cfg;
-  return 0;
+  static const int small = config_of(128, 1, 4), medium = config_of(64, 2, 4), large = config_of(64, 4, 8);
+  return W < 6.0e6 ? small : (W < 1.2e8 ? medium : large);
 }
 
 // Schedule of the real/Kelvin pair items in the fused graph: forced, else the size class's
@@ -1665,7 +1738,7 @@ int hsma_workspace_size(hsma_t* h, int64_t n, size_t* bytes)
 {
   if (!h || !bytes || n < 0 || n > (int64_t)INT32_MAX / 4) return set_err(h, HSMA_E_INVALID_ARG, "bad argument");
   const int cfg = h->e->prec == HSMA_FP64 ? 0 : h->e->choose_config({n});
-  *bytes = h->e->make_layout({n}, cfg).bytes;
+  *bytes = h->e->make_layout({n}, cfg, true).bytes;
   return HSMA_OK;
 }
 

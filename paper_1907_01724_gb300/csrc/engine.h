@@ -51,6 +51,9 @@ struct Layout {
   std::vector<int2> selrng;   // their reduce-item ranges
   size_t o_sel = 0, o_selrng = 0;
   int cfg = 0, maxP = 1, pmax = 0, mom_stride = 3, pair_grid = 1;
+  int TBf = 1;               // targets per field item
+  size_t n4 = 0, n4f = 0;    // pair and field items
+  bool field_items = false;  // it4f, it4fx made and uploaded
   int64_t totN = 0, totM = 0, totP = 0, totMn = 0, totMom = 0, totPart = 0;
   size_t o_sys = 0, o_Mn = 0, o_rec_a = 0, o_rec_b = 0, o_sect = 0, o_inv_np1 = 0, o_xyz = 0, o_q = 0;
   size_t o_rec_a2 = 0, o_rec_b2 = 0, o_sect2 = 0, o_mtab = 0;
@@ -78,7 +81,10 @@ class Engine {
  public:
   ~Engine();
   int init(int dev, void* user_stream, int precision);
-  Layout make_layout(const std::vector<int64_t>& ns, int cfg) const;
+  Layout make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_only = false) const;
+  void sort_items(const Layout& L, std::vector<int4>& items, bool field) const;
+  int split_items(const Layout& L, std::vector<int4>& items) const;
+  int make_field_items();
   int set_sizes(const std::vector<int64_t>& ns);
   int attach(void* ptr, size_t bytes);
   int build(const double* xyz, const double* q, bool device_inputs);

@@ -719,7 +719,7 @@ int hsma_server_load(hsma_server_t* s, const int64_t* n, const double* xyz, cons
     // device footprint of the chain on its own
     Engine& e = *s->e;
     e.spec = {s->specs[c]};
-    s->footprint[c] = e.make_layout({n[c]}, e.prec == HSMA_FP64 ? 0 : e.choose_config({n[c]})).bytes;
+    s->footprint[c] = e.make_layout({n[c]}, e.prec == HSMA_FP64 ? 0 : e.choose_config({n[c]}), true).bytes;
     off += n[c];
   }
   int rc = admit(s, admitted);

@@ -3,6 +3,7 @@ dispatch rule, against the FP64 oracle or against an exact relation."""
 import numpy as np
 import pytest
 
+import oracle
 from paper_1907_01724_gb300 import api, inputs
 
 pytestmark = pytest.mark.gpu
@@ -20,3 +21,20 @@ def test_fp64_potentials_scale_with_the_cavity(n, scale):
            for a in (1.0, scale)]
     # every operation scales exactly except through the range of exponents: rounding of a few sums
     assert np.linalg.norm(phi[1] * scale - phi[0]) <= 1e-12 * np.linalg.norm(phi[0])
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 129, 1437, 1438, 7428, 7429])
+def test_default_tile_configurations(n):
+    """The tile configuration chosen without tuning, on both sides of the rule's lines (M = 1000),
+    and the layer's term at charges next to the interface: potentials and fields, 1e-6 norm-wise
+    (the FP32 path's bound)."""
+    rng = np.random.default_rng(190800 + n)
+    k = (n + 3) // 4
+    xyz = np.concatenate([inputs.shell(rng, k, 1.0, 0.02), inputs.uniform_ball(rng, n - k, 1.0)])
+    q = rng.choice([-1.0, 1.0], n)
+    P = oracle.make_params(a=1.0, eps1=2.0, eps2=80.0, kappa=1.5, p=12, M=1000)
+    ref, E = oracle.hsma(P, xyz, q)["phi"], oracle.field(P, xyz, q)["E"]
+    h = api.hsma_create(1.0, 2.0, 80.0, 1.5, api.hsma_default_params(p=12, M=1000))
+    api.hsma_build_sources(h, xyz, q)
+    assert np.linalg.norm(api.hsma_potential(h) - ref) <= 1e-6 * np.linalg.norm(ref)
+    assert np.linalg.norm(api.hsma_field(h) - E) <= 1e-6 * np.linalg.norm(E)
