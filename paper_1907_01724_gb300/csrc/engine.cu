@@ -617,11 +617,11 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_o
   L.o_sel = take(sizeof(int) * (size_t)nsys);
   L.o_selrng = take(sizeof(int2) * (size_t)nsys);
   if (L.tree) {
-    const size_t nodes = (size_t)tree_node_count(L.tL), nm = (size_t)tree_nm(L.tP);
+    const size_t nodes = (size_t)tree_node_count(L.tL), nq = (size_t)tree_nq(L.tP);
     L.o_tnode = take(sizeof(int2) * nodes);
     L.o_tgeo = take(sizeof(float4) * 2 * nodes);
     L.o_tbox = take(sizeof(float4) * 4 * nodes);
-    L.o_tmom = take(sizeof(float2) * 2 * nodes * nm);
+    L.o_tmom = take(sizeof(float4) * 2 * nodes * nq);
     L.o_tfarp = take(sizeof(float2) * kFarBlocks * (size_t)tree_nm(kFarOrder));
     L.o_tfarL = take(sizeof(float2) * (size_t)tree_nm(kFarOrder));
     L.o_tctr = take(16);
@@ -849,14 +849,14 @@ TreeView Engine::tree_view() const
   t.node = (int2*)(b + L.o_tnode);
   t.geo = (float4*)(b + L.o_tgeo);
   t.box = (float4*)(b + L.o_tbox);
-  t.mom = (float2*)(b + L.o_tmom);
+  t.mom = (float4*)(b + L.o_tmom);
   t.farp = (float2*)(b + L.o_tfarp);
   t.farL = (float2*)(b + L.o_tfarL);
   t.ctr = (unsigned int*)(b + L.o_tctr);
   t.L = L.tL;
   t.key_lv = L.sd[0].key_lv;
   t.P = L.tP;
-  t.cmin = (L.tP + 1) * (L.tP + 1) / 3;  // ~850 instructions per evaluation against ~16 per pair
+  t.cmin = (L.tP + 1) * (L.tP + 1) / 3;  // ~400 instructions per evaluation against 7 a pair
   t.theta = (float)far_theta;
   t.log_eps = (float)(std::log(0.1) + (L.tP + 1) * std::log(far_theta > 0.0 ? far_theta : 0.5));
   const double a = spec[0].a;

@@ -38,16 +38,19 @@
 //   R_m^m = R_{m-1}^{m-1} (x + i y) / (2m),     R_n^m = [(2n-1) z R_{n-1}^m - r^2 R_{n-2}^m] / (n^2 - m^2),
 //   I_m^m = I_{m-1}^{m-1} (2m-1)(x + i y) / r^2, I_n^m = [(2n-1) z I_{n-1}^m - ((n-1)^2 - m^2) I_{n-2}^m] / r^2,
 // with R_0^0 = 1, I_0^0 = 1/r.  A node of centre c and radius rho stores the moments
-// M_n^m = sum_j Q_j conj(R_n^m((y_j - c)/rho)) and gives phi(x) = (1/rho) sum w_m Re(M_n^m I_n^m((x - c)/rho))
+// M_n^m = sum_j Q_j conj(R_n^m((y_j - c)/s)) in units of s, the power of two above rho (so that 1/s is
+// exact and costs an integer operation), and gives phi(x) = (1/s) sum w_m Re(M_n^m I_n^m((x - c)/s))
 // (w_0 = 1, w_m = 2).  The far images give L_n^m = sum_j Q_j conj(I_n^m(y_j/a)) and
 // phi(x) = (1/a) sum w_m Re(L_n^m R_n^m(x/a)) inside the cavity.
-// Shift of a child's moments (centre c', radius rho') to the parent (c, rho): with b = (c' - c)/rho,
-// s = rho'/rho, and the solid harmonics continued to m < 0 in the Condon-Shortley convention
+// Shift of a child's moments (centre c', unit s') to the parent (c, s0): with b = (c' - c)/s0,
+// s = s'/s0, and the solid harmonics continued to m < 0 in the Condon-Shortley convention
 // (X_n^{-m} = conj(X_n^m), X_n^m -> (-1)^m X_n^m for m > 0), the addition theorem
 // R_n^m(u + v) = sum_{j,k} R_j^k(u) R_{n-j}^{m-k}(v) of the regular harmonics gives
 //   M_n^m = (-1)^m sum_{j <= n} s^j sum_k A_j^k conj(B_{n-j}^{m-k}),
 //   A_j^k = (-1)^k M'_j^k (k >= 0), conj(M'_j^{-k}) (k < 0);  B_l^t = (-1)^t R_l^t(b) (t >= 0), conj(R_l^{-t}(b)) (t < 0).
-// Moments are stored by column: (n, m) at m (P + 1) - m (m - 1)/2 + (n - m).
+// Moments are stored by column pair: (n, 2k) and (n, 2k + 1) side by side as (Re, Re, Im, Im), k
+// outermost, rows n = 2k..P (the odd column's entry at n = 2k is zero), which is how the evaluation
+// reads them; the far-image expansion by column, (n, m) at m (P + 1) - m (m - 1)/2 + (n - m).
 #include <algorithm>
 #include <cmath>
 
@@ -58,6 +61,27 @@
 namespace hsma {
 
 __host__ __device__ constexpr int tree_col(int P, int m) { return m * (P + 1) - m * (m - 1) / 2; }
+// entry (row n of pair k) of a node's moments
+__host__ __device__ constexpr int tree_pair(int P, int k, int n) { return k * (P + 2 - k) + n - 2 * k; }
+
+__device__ __forceinline__ void put_moment(float4* M, int P, int n, int m, float re, float im)
+{
+  float* e = reinterpret_cast<float*>(M + tree_pair(P, m >> 1, n)) + (m & 1);
+  e[0] = re;
+  e[2] = im;
+  if ((m & 1) == 0 && n == m) e[1] = e[3] = 0.f;  // the odd column starts a row later
+}
+__device__ __forceinline__ float2 get_moment(const float4* M, int P, int n, int m)
+{
+  const float* e = reinterpret_cast<const float*>(M + tree_pair(P, m >> 1, n)) + (m & 1);
+  return make_float2(e[0], e[2]);
+}
+
+// 1/s of a node of radius rho > 0: s = 2^(e + 1) for rho in [2^e, 2^(e + 1))
+__device__ __forceinline__ float inv_unit(float rho)
+{
+  return __int_as_float(0x7e800000 - (__float_as_int(rho) & 0x7f800000));
+}
 
 // Whether a Kelvin record lies beyond kFarImageRel a (its high part, rounded without contraction,
 // so that every kernel classifies a record the same way).
@@ -113,7 +137,7 @@ constexpr int kLeafWarps = 4;
 template <int P>
 __global__ __launch_bounds__(32 * kLeafWarps) void k_tree_leaf(TreeView t)
 {
-  constexpr int NM = tree_nm(P);
+  constexpr int NQ = tree_nq(P);
   const int lane = threadIdx.x & 31;
   const long long c = (long long)blockIdx.x * kLeafWarps + (threadIdx.x >> 5);
   if (c >= (1LL << (3 * t.L))) return;  // whole warps
@@ -145,14 +169,14 @@ __global__ __launch_bounds__(32 * kLeafWarps) void k_tree_leaf(TreeView t)
     mx2 = warp_max(mx2);
     float4* geo = t.geo + (long long)tr * nodes + g;
     float4* bx = t.box + 2 * ((long long)tr * nodes + g);
-    float2* M = t.mom + ((long long)tr * nodes + g) * NM;
+    float4* M = t.mom + ((long long)tr * nodes + g) * NQ;
     if (!(mn0 <= mx0)) {
       if (lane == 0) {
         *geo = make_float4(0.f, 0.f, 0.f, -1.f);
         bx[0] = make_float4(3.0e38f, 3.0e38f, 3.0e38f, 0.f);
         bx[1] = make_float4(-3.0e38f, -3.0e38f, -3.0e38f, 0.f);
       }
-      for (int k = lane; k < NM; k += 32) M[k] = make_float2(0.f, 0.f);
+      for (int k = lane; k < NQ; k += 32) M[k] = make_float4(0.f, 0.f, 0.f, 0.f);
       continue;
     }
     const float cx = 0.5f * (mn0 + mx0), cy = 0.5f * (mn1 + mx1), cz = 0.5f * (mn2 + mx2);
@@ -170,7 +194,7 @@ __global__ __launch_bounds__(32 * kLeafWarps) void k_tree_leaf(TreeView t)
       bx[0] = make_float4(mn0, mn1, mn2, 0.f);
       bx[1] = make_float4(mx0, mx1, mx2, 0.f);
     }
-    const float ir = 1.f / rho;
+    const float ir = inv_unit(rho);
 #pragma unroll
     for (int m = 0; m <= P; ++m) {
       float cr[P + 1], ci[P + 1];
@@ -209,15 +233,20 @@ __global__ __launch_bounds__(32 * kLeafWarps) void k_tree_leaf(TreeView t)
 #pragma unroll
       for (int k = 0; k <= P - m; ++k) {
         const float sr = warp_sum(cr[k]), si = warp_sum(ci[k]);
-        if (lane == 0) M[tree_col(P, m) + k] = make_float2(sr, si);
+        if (lane == 0) put_moment(M, P, m + k, m, sr, si);
       }
     }
   }
 }
 
 // ---------------------------------------------------------------------------------------
-// Upward pass, level l < L: a warp per node, from its 8 children (level l + 1).
-constexpr int kUpWarps = 4;
+// Upward pass, level l < L: a block per node and tree, a warp per child (order 16: per two
+// children, for the shared memory), the children's shifted moments summed in child order.  Bound by
+// the latency of a child's chain (stage, 91 sums of up to 91 products): a warp that walked the
+// eight children took 250 us at each of the levels of 64 and 512 nodes (N = 1e5: the build and the
+// rest of the step 1041 us, 576 us so).
+template <int P>
+constexpr int up_warps() { return P > 12 ? 4 : 8; }
 template <int P>
 __device__ __forceinline__ void decode_nm(int idx, int& n, int& m)
 {
@@ -227,21 +256,61 @@ __device__ __forceinline__ void decode_nm(int idx, int& n, int& m)
 }
 
 template <int P>
-__global__ __launch_bounds__(32 * kUpWarps) void k_tree_up(TreeView t, int l)
+__global__ __launch_bounds__(32 * (P > 12 ? 4 : 8)) void k_tree_up(TreeView t, int l)
 {
-  constexpr int NM = tree_nm(P);
+  constexpr int NM = tree_nm(P), NQ = tree_nq(P);
+  constexpr int W = P > 12 ? 4 : 8;
   constexpr int OUT = (NM + 31) / 32;
   constexpr int KW = 2 * P + 1;  // k = -P..P
   // per warp, for the child being shifted: A[j][k] = s^j A_j^k and B[l][t] = conj(B_l^t), dense
   // over -P <= k, t <= P (entries with |k| > j or |t| > l are never read)
-  __shared__ float2 sAd[kUpWarps][(P + 1) * KW], sBd[kUpWarps][(P + 1) * KW];
-  __shared__ float sPow[kUpWarps][P + 1];
+  __shared__ float2 sAd[W][(P + 1) * KW], sBd[W][(P + 1) * KW];
+  __shared__ float sPow[W][P + 1];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const long long c = (long long)blockIdx.x * kUpWarps + w;
-  if (c >= (1LL << (3 * l))) return;  // whole warps
+  const long long c = blockIdx.x;
+  const int tr = blockIdx.y;
   const long long nodes = tree_node_count(t.L);
   const long long g = tree_node_index(l, c);
   const long long g0 = tree_node_index(l + 1, 8 * c);
+  const long long base = (long long)tr * nodes;
+  float4 cg = make_float4(0.f, 0.f, 0.f, -1.f);
+  float4 bmn = make_float4(3.0e38f, 3.0e38f, 3.0e38f, 0.f), bmx = make_float4(-3.0e38f, -3.0e38f, -3.0e38f, 0.f);
+  if (lane < 8) {
+    cg = t.geo[base + g0 + lane];
+    if (cg.w >= 0.f) {
+      bmn = t.box[2 * (base + g0 + lane)];
+      bmx = t.box[2 * (base + g0 + lane) + 1];
+    }
+  }
+  const bool ne = lane < 8 && cg.w >= 0.f;
+  const unsigned any = __ballot_sync(0xffffffffu, ne);
+  float4* geo = t.geo + base + g;
+  float4* bx = t.box + 2 * (base + g);
+  float4* M = t.mom + (base + g) * NQ;
+  if (!any) {  // (the same in every warp)
+    if (threadIdx.x == 0) {
+      *geo = make_float4(0.f, 0.f, 0.f, -1.f);
+      bx[0] = make_float4(3.0e38f, 3.0e38f, 3.0e38f, 0.f);
+      bx[1] = make_float4(-3.0e38f, -3.0e38f, -3.0e38f, 0.f);
+    }
+    for (int k = threadIdx.x; k < NQ; k += blockDim.x) M[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    return;
+  }
+  const float mn0 = warp_min(bmn.x), mn1 = warp_min(bmn.y), mn2 = warp_min(bmn.z);
+  const float mx0 = warp_max(bmx.x), mx1 = warp_max(bmx.y), mx2 = warp_max(bmx.z);
+  const float cx = 0.5f * (mn0 + mx0), cy = 0.5f * (mn1 + mx1), cz = 0.5f * (mn2 + mx2);
+  float rr = 0.f;
+  if (ne) {
+    const float dx = cg.x - cx, dy = cg.y - cy, dz = cg.z - cz;
+    rr = sqrtf(dx * dx + dy * dy + dz * dz) + cg.w;
+  }
+  const float rho = warp_max(rr) * 1.000001f;
+  if (threadIdx.x == 0) {
+    *geo = make_float4(cx, cy, cz, rho);
+    bx[0] = make_float4(mn0, mn1, mn2, 0.f);
+    bx[1] = make_float4(mx0, mx1, mx2, 0.f);
+  }
+  const float irp = inv_unit(rho);
   int on[OUT], om[OUT];
 #pragma unroll
   for (int q = 0; q < OUT; ++q) {
@@ -253,131 +322,107 @@ __global__ __launch_bounds__(32 * kUpWarps) void k_tree_up(TreeView t, int l)
       om[q] = 0;
     }
   }
-  for (int tr = 0; tr < 2; ++tr) {
-    const long long base = (long long)tr * nodes;
-    float4 cg = make_float4(0.f, 0.f, 0.f, -1.f);
-    float4 bmn = make_float4(3.0e38f, 3.0e38f, 3.0e38f, 0.f), bmx = make_float4(-3.0e38f, -3.0e38f, -3.0e38f, 0.f);
-    if (lane < 8) {
-      cg = t.geo[base + g0 + lane];
-      if (cg.w >= 0.f) {
-        bmn = t.box[2 * (base + g0 + lane)];
-        bmx = t.box[2 * (base + g0 + lane) + 1];
-      }
-    }
-    const bool ne = lane < 8 && cg.w >= 0.f;
-    const unsigned any = __ballot_sync(0xffffffffu, ne);
-    float4* geo = t.geo + base + g;
-    float4* bx = t.box + 2 * (base + g);
-    float2* M = t.mom + (base + g) * NM;
-    if (!any) {
-      if (lane == 0) {
-        *geo = make_float4(0.f, 0.f, 0.f, -1.f);
-        bx[0] = make_float4(3.0e38f, 3.0e38f, 3.0e38f, 0.f);
-        bx[1] = make_float4(-3.0e38f, -3.0e38f, -3.0e38f, 0.f);
-      }
-      for (int k = lane; k < NM; k += 32) M[k] = make_float2(0.f, 0.f);
-      continue;
-    }
-    const float mn0 = warp_min(bmn.x), mn1 = warp_min(bmn.y), mn2 = warp_min(bmn.z);
-    const float mx0 = warp_max(bmx.x), mx1 = warp_max(bmx.y), mx2 = warp_max(bmx.z);
-    const float cx = 0.5f * (mn0 + mx0), cy = 0.5f * (mn1 + mx1), cz = 0.5f * (mn2 + mx2);
-    float rr = 0.f;
-    if (ne) {
-      const float dx = cg.x - cx, dy = cg.y - cy, dz = cg.z - cz;
-      rr = sqrtf(dx * dx + dy * dy + dz * dz) + cg.w;
-    }
-    const float rho = warp_max(rr) * 1.000001f;
-    if (lane == 0) {
-      *geo = make_float4(cx, cy, cz, rho);
-      bx[0] = make_float4(mn0, mn1, mn2, 0.f);
-      bx[1] = make_float4(mx0, mx1, mx2, 0.f);
-    }
-    const float irp = 1.f / rho;
-    float accr[OUT], acci[OUT];
+  float2 acc[8 / W][OUT];
 #pragma unroll
-    for (int q = 0; q < OUT; ++q) accr[q] = acci[q] = 0.f;
-    for (int k = 0; k < 8; ++k) {
-      if (!((any >> k) & 1u)) continue;  // uniform
-      const float kx = __shfl_sync(0xffffffffu, cg.x, k), ky = __shfl_sync(0xffffffffu, cg.y, k);
-      const float kz = __shfl_sync(0xffffffffu, cg.z, k), kr = __shfl_sync(0xffffffffu, cg.w, k);
-      const float s = kr * irp;
-      const float bxv = (kx - cx) * irp, byv = (ky - cy) * irp, bzv = (kz - cz) * irp;
-      const float2* Mc = t.mom + (base + g0 + k) * NM;
-      if (lane <= P) {
-        // column m = lane of R(b) into B (both signs of t), and s^lane
-        const int m = lane;
-        const float r2 = bxv * bxv + byv * byv + bzv * bzv;
-        float dr = 1.f, di = 0.f;
-        for (int j = 1; j <= m; ++j) {
-          const float f = 0.5f / (float)j;
-          const float nr = (dr * bxv - di * byv) * f;
-          di = (dr * byv + di * bxv) * f;
-          dr = nr;
-        }
-        const float sgn = (m & 1) ? -1.f : 1.f;
-        float p0r = 0.f, p0i = 0.f, p1r = dr, p1i = di;
-        for (int nn = m; nn <= P; ++nn) {
-          if (nn > m) {
-            const float A = (float)(2 * nn - 1) * bzv;
-            const float inv = 1.f / (float)(nn * nn - m * m);
-            const float qr = (A * p1r - r2 * p0r) * inv, qi = (A * p1i - r2 * p0i) * inv;
-            p0r = p1r;
-            p0i = p1i;
-            p1r = qr;
-            p1i = qi;
-          }
-          // conj(B_nn^m) = (-1)^m conj(R_nn^m); conj(B_nn^-m) = R_nn^m
-          sBd[w][nn * KW + P + m] = make_float2(sgn * p1r, -sgn * p1i);
-          if (m > 0) sBd[w][nn * KW + P - m] = make_float2(p1r, p1i);
-        }
-        float sp = 1.f;
-        for (int j = 0; j < m; ++j) sp *= s;
-        sPow[w][m] = sp;
-      }
-      __syncwarp();
-      for (int e = lane; e < (P + 1) * KW; e += 32) {
-        const int j = e / KW, kk = e - j * KW - P;
-        if (kk > j || -kk > j) continue;
-        const int ka = kk >= 0 ? kk : -kk;
-        float2 A = Mc[tree_col(P, ka) + j - ka];
-        if (kk >= 0) {
-          if (kk & 1) A = make_float2(-A.x, -A.y);
-        } else {
-          A.y = -A.y;
-        }
-        const float sj = sPow[w][j];
-        sAd[w][e] = make_float2(sj * A.x, sj * A.y);
-      }
-      __syncwarp();
+  for (int kk = 0; kk < 8 / W; ++kk) {
+    const int k = w * (8 / W) + kk;
 #pragma unroll
-      for (int q = 0; q < OUT; ++q) {
-        const int n = on[q], m = om[q];
-        if (n < 0) continue;
-        float ar = 0.f, ai = 0.f;
-        for (int j = 0; j <= n; ++j) {
-          const int l2 = n - j;
-          const int k0 = max(-j, m - l2), k1 = min(j, m + l2);
-          const float2* Aj = &sAd[w][j * KW + P];
-          const float2* Bl = &sBd[w][l2 * KW + P + m];  // Bl[-kk] = conj(B_{l2}^{m-kk})
-          for (int kk = k0; kk <= k1; ++kk) {
-            const float2 A = Aj[kk], B = Bl[-kk];
-            ar = fmaf(A.x, B.x, ar);
-            ar = fmaf(-A.y, B.y, ar);
-            ai = fmaf(A.x, B.y, ai);
-            ai = fmaf(A.y, B.x, ai);
-          }
-        }
-        accr[q] += ar;
-        acci[q] += ai;
+    for (int q = 0; q < OUT; ++q) acc[kk][q] = make_float2(0.f, 0.f);
+    if (!((any >> k) & 1u)) continue;  // whole warps
+    const float kx = __shfl_sync(0xffffffffu, cg.x, k), ky = __shfl_sync(0xffffffffu, cg.y, k);
+    const float kz = __shfl_sync(0xffffffffu, cg.z, k), kr = __shfl_sync(0xffffffffu, cg.w, k);
+    const float s = irp / inv_unit(kr);
+    const float bxv = (kx - cx) * irp, byv = (ky - cy) * irp, bzv = (kz - cz) * irp;
+    const float4* Mc = t.mom + (base + g0 + k) * NQ;
+    if (lane <= P) {
+      // column m = lane of R(b) into B (both signs of t), and s^lane
+      const int m = lane;
+      const float r2 = bxv * bxv + byv * byv + bzv * bzv;
+      float dr = 1.f, di = 0.f;
+      for (int j = 1; j <= m; ++j) {
+        const float f = 0.5f / (float)j;
+        const float nr = (dr * bxv - di * byv) * f;
+        di = (dr * byv + di * bxv) * f;
+        dr = nr;
       }
-      __syncwarp();
+      const float sgn = (m & 1) ? -1.f : 1.f;
+      float p0r = 0.f, p0i = 0.f, p1r = dr, p1i = di;
+      for (int nn = m; nn <= P; ++nn) {
+        if (nn > m) {
+          const float A = (float)(2 * nn - 1) * bzv;
+          const float inv = 1.f / (float)(nn * nn - m * m);
+          const float qr = (A * p1r - r2 * p0r) * inv, qi = (A * p1i - r2 * p0i) * inv;
+          p0r = p1r;
+          p0i = p1i;
+          p1r = qr;
+          p1i = qi;
+        }
+        // conj(B_nn^m) = (-1)^m conj(R_nn^m); conj(B_nn^-m) = R_nn^m
+        sBd[w][nn * KW + P + m] = make_float2(sgn * p1r, -sgn * p1i);
+        if (m > 0) sBd[w][nn * KW + P - m] = make_float2(p1r, p1i);
+      }
+      float sp = 1.f;
+      for (int j = 0; j < m; ++j) sp *= s;
+      sPow[w][m] = sp;
     }
+    __syncwarp();
+    for (int e = lane; e < (P + 1) * KW; e += 32) {
+      const int j = e / KW, kq = e - j * KW - P;
+      if (kq > j || -kq > j) continue;
+      const int ka = kq >= 0 ? kq : -kq;
+      float2 A = get_moment(Mc, P, j, ka);
+      if (kq >= 0) {
+        if (kq & 1) A = make_float2(-A.x, -A.y);
+      } else {
+        A.y = -A.y;
+      }
+      const float sj = sPow[w][j];
+      sAd[w][e] = make_float2(sj * A.x, sj * A.y);
+    }
+    __syncwarp();
 #pragma unroll
     for (int q = 0; q < OUT; ++q) {
-      if (on[q] < 0) continue;
-      const float sg = (om[q] & 1) ? -1.f : 1.f;
-      M[lane + 32 * q] = make_float2(sg * accr[q], sg * acci[q]);
+      const int n = on[q], m = om[q];
+      if (n < 0) continue;
+      float ar = 0.f, ai = 0.f;
+      for (int j = 0; j <= n; ++j) {
+        const int l2 = n - j;
+        const int k0 = max(-j, m - l2), k1 = min(j, m + l2);
+        const float2* Aj = &sAd[w][j * KW + P];
+        const float2* Bl = &sBd[w][l2 * KW + P + m];  // Bl[-kq] = conj(B_{l2}^{m-kq})
+        for (int kq = k0; kq <= k1; ++kq) {
+          const float2 A = Aj[kq], B = Bl[-kq];
+          ar = fmaf(A.x, B.x, ar);
+          ar = fmaf(-A.y, B.y, ar);
+          ai = fmaf(A.x, B.y, ai);
+          ai = fmaf(A.y, B.x, ai);
+        }
+      }
+      acc[kk][q] = make_float2(ar, ai);
     }
+    __syncwarp();
+  }
+  // the children in order, through the warps' own (spent) tables
+  __syncthreads();
+  float2* sum = &sAd[0][0];  // [8][NM]
+  static_assert(8 * tree_nm(P) <= W * (P + 1) * KW, "the children's moments fit the tables");
+#pragma unroll
+  for (int kk = 0; kk < 8 / W; ++kk)
+#pragma unroll
+    for (int q = 0; q < OUT; ++q)
+      if (on[q] >= 0) sum[(w * (8 / W) + kk) * NM + lane + 32 * q] = acc[kk][q];
+  __syncthreads();
+  for (int i = threadIdx.x; i < NM; i += blockDim.x) {
+    float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      v.x += sum[k * NM + i].x;
+      v.y += sum[k * NM + i].y;
+    }
+    int n, m;
+    decode_nm<P>(i, n, m);
+    const float sg = (m & 1) ? -1.f : 1.f;
+    put_moment(M, P, n, m, sg * v.x, sg * v.y);
   }
 }
 
@@ -477,106 +522,103 @@ __global__ __launch_bounds__(32 * kFarWarps) void k_tree_far(TreeView t)
 
 // ---------------------------------------------------------------------------------------
 // Evaluation.
-// phi at target (th, tl) of a node's moments M (stored to order P; centre and radius gc), the
-// series truncated at order Q <= P.
-template <int P, int Q>
-__device__ __forceinline__ float m2p(const float2* __restrict__ M, float4 gc, float4 th, float4 tl)
+// phi at target (th, tl) of a node's moments M (shared memory, stored to order P; centre and radius
+// gc), the series truncated at order q <= P.
+//
+// I_n^m = Q_n^m z^m with z = (x + i y)/r^2 and a real recurrence in n: Q_m^m = (2m-1)!!/r,
+// Q_n^m = (2n-1) w Q_{n-1}^m - ((n-1)^2 - m^2) Q_{n-2}^m / r^2, w = z/r^2.  So the column sums
+// C_m = sum_n M_n^m Q_n^m take, per coefficient, the recurrence once (not for a real and an imaginary
+// part) and two multiply-adds, and z enters in one Horner sum of 2 Re sum_m C_m z^m.  Packed FP32 over
+// the columns 2k, 2k + 1 (FFMA2 / FMUL2): per two coefficients one 16-byte shared load, the two
+// factors of Q_{n-2}, three operations of the recurrence and two of the sums -- 3.5 instructions a
+// coefficient where the recurrence on (Re, Im) took 5.  The columns run in two groups so that the state
+// (two rows and the sums) fits the registers of 24 warps per SM.  The evaluation is issue-bound
+// (76 % of the slots): with this series, the direct sums relative to the node's centre and one
+// reduction for the three tests of a node it takes 1.75 ms at N = 1e5 and 19.9 ms at N = 1e6 (theta =
+// 0.5, order 12; 2.47 and 24.2 ms before), at the same error (7.6e-8 at N = 1e5).
+template <int P, int K0, int K1>
+__device__ __forceinline__ void series_group(const float4* M, float wz, float i2, float ri, int q,
+                                             float2 (&CR)[K1 - K0], float2 (&CI)[K1 - K0])
 {
-  const float ir = 1.f / gc.w;
-  const float ux = ((th.x - gc.x) + tl.x) * ir, uy = ((th.y - gc.y) + tl.y) * ir, uz = ((th.z - gc.z) + tl.z) * ir;
-  const float r2 = ux * ux + uy * uy + uz * uz;
-  const float i2 = __frcp_rn(r2);
-  const float px = ux * i2, py = uy * i2, wz = uz * i2;
-  float dr = rsqrt_mufu(r2), di = 0.f;  // I_0^0
-  float acc = 0.f;
-  {
-    // m = 0: the column is real (written out: IEEE arithmetic does not let the compiler drop
-    // the zero imaginary parts)
-    float p0 = 0.f, p1 = dr;
-    float col = __ldg(M).x * dr;
+  constexpr int NK = K1 - K0;
+  float2 a[NK], b[NK];
 #pragma unroll
-    for (int nn = 1; nn <= Q; ++nn) {
-      const float A = (float)(2 * nn - 1) * wz, B = (float)((nn - 1) * (nn - 1)) * i2;
-      const float q = A * p1 - B * p0;
-      col = fmaf(__ldg(M + nn).x, q, col);
-      p0 = p1;
-      p1 = q;
-    }
-    acc = col;
-  }
+  for (int k = 0; k < NK; ++k) a[k] = b[k] = CR[k] = CI[k] = make_float2(0.f, 0.f);
 #pragma unroll
-  for (int m = 1; m <= Q; ++m) {
-    {
-      const float f = (float)(2 * m - 1);
-      const float nr = f * (dr * px - di * py);
-      di = f * (dr * py + di * px);
-      dr = nr;
-    }
-    const float2* Mc = M + tree_col(P, m);
-    float2 mm = __ldg(Mc);
-    float col = mm.x * dr - mm.y * di;
-    float p0r = 0.f, p0i = 0.f, p1r = dr, p1i = di;
-#pragma unroll
-    for (int nn = m + 1; nn <= Q; ++nn) {
-      const float A = (float)(2 * nn - 1) * wz, B = (float)((nn - 1) * (nn - 1) - m * m) * i2;
-      const float qr = A * p1r - B * p0r, qi = A * p1i - B * p0i;
-      mm = __ldg(Mc + (nn - m));
-      col = fmaf(mm.x, qr, col);
-      col = fmaf(-mm.y, qi, col);
-      p0r = p1r;
-      p0i = p1i;
-      p1r = qr;
-      p1i = qi;
-    }
-    acc = fmaf(2.f, col, acc);
-  }
-  return acc * ir;
-}
-
-// The same sum row by row (n outer), truncated at a runtime order q <= P: rows n and n - 1 of
-// I_n^m stay in registers, so one code path serves every order (the nodes far beyond the opening
-// criterion need far fewer terms for the same truncation bound).
-template <int P>
-__device__ __forceinline__ float m2p_rows(const float2* M, float4 gc, float4 th, float4 tl, int q)
-{
-  const float ir = 1.f / gc.w;
-  const float ux = ((th.x - gc.x) + tl.x) * ir, uy = ((th.y - gc.y) + tl.y) * ir, uz = ((th.z - gc.z) + tl.z) * ir;
-  const float r2 = ux * ux + uy * uy + uz * uz;
-  const float i2 = __frcp_rn(r2);
-  const float px = ux * i2, py = uy * i2, wz = uz * i2;
-  // rows n - 1 (a) and n - 2 (b) as (re, im) pairs: the recurrence's complex-by-real products
-  // and the dot product with the (re, -im) moments as packed FP32 (FFMA2 / FMUL2)
-  float2 a[P + 1], b[P + 1];
-#pragma unroll
-  for (int m = 0; m <= P; ++m) a[m] = b[m] = make_float2(0.f, 0.f);
-  a[0].x = rsqrt_mufu(r2);  // I_0^0
-  float acc0 = M[0].x * a[0].x;       // m = 0 terms
-  float2 acc1 = make_float2(0.f, 0.f);  // m > 0 terms (weight 2): the re re and -im im parts
-#pragma unroll
-  for (int n = 1; n <= P; ++n) {
+  for (int n = 2 * K0; n <= P; ++n) {
     if (n > q) break;
     const float A = (float)(2 * n - 1) * wz;
     const float2 A2 = make_float2(A, A);
-    // the new diagonal I_n^n from I_{n-1}^{n-1}
-    const float f = (float)(2 * n - 1);
-    const float dr = f * (a[n - 1].x * px - a[n - 1].y * py), di = f * (a[n - 1].x * py + a[n - 1].y * px);
 #pragma unroll
-    for (int m = 0; m < n; ++m) {
-      const float nB = (float)(m * m - (n - 1) * (n - 1)) * i2;  // -B (zero for m = n - 1)
-      const float2 nv = __ffma2_rn(make_float2(nB, nB), b[m], __fmul2_rn(A2, a[m]));
-      b[m] = a[m];
-      a[m] = nv;
-      const float2 mm = M[tree_col(P, m) + (n - m)];
-      if (m == 0)
-        acc0 = fmaf(mm.x, nv.x, acc0);
-      else
-        acc1 = __ffma2_rn(mm, nv, acc1);
+    for (int k = 0; k < NK; ++k) {
+      const int m = 2 * (K0 + k);
+      if (n < m) continue;
+      float2 v;
+      if (n == m) {
+        float f = ri;  // (2m - 1)!! / r
+#pragma unroll
+        for (int j = 1; j < 2 * m; j += 2) f *= (float)j;
+        v = make_float2(f, 0.f);
+      } else {
+        const float2 B2 = make_float2((float)(m * m - (n - 1) * (n - 1)) * i2,
+                                      (float)((m + 1) * (m + 1) - (n - 1) * (n - 1)) * i2);
+        v = __ffma2_rn(B2, b[k], __fmul2_rn(A2, a[k]));
+        if (n == m + 1) {
+          float f = ri;
+#pragma unroll
+          for (int j = 1; j < 2 * (m + 1); j += 2) f *= (float)j;
+          v.y = f;
+        }
+      }
+      b[k] = a[k];
+      a[k] = v;
+      const float4 mm = M[tree_pair(P, K0 + k, n)];
+      CR[k] = __ffma2_rn(make_float2(mm.x, mm.y), v, CR[k]);
+      CI[k] = __ffma2_rn(make_float2(mm.z, mm.w), v, CI[k]);
     }
-    b[n] = make_float2(0.f, 0.f);
-    a[n] = make_float2(dr, di);
-    acc1 = __ffma2_rn(M[tree_col(P, n)], a[n], acc1);
   }
-  return fmaf(2.f, acc1.x + acc1.y, acc0) * ir;
+}
+
+// S <- S z + C
+__device__ __forceinline__ void horner(float& sr, float& si, float zx, float zy, float cr, float ci)
+{
+  const float nr = fmaf(sr, zx, fmaf(-si, zy, cr));
+  si = fmaf(sr, zy, fmaf(si, zx, ci));
+  sr = nr;
+}
+
+template <int P>
+__device__ __forceinline__ float m2p(const float4* M, float4 gc, float4 th, float4 tl, int q)
+{
+  constexpr int KP = P / 2 + 1;              // column pairs
+  constexpr int KS = P <= 8 ? KP : P / 4;    // first pair of the second group
+  const float ir = inv_unit(gc.w);
+  const float ux = ((th.x - gc.x) + tl.x) * ir, uy = ((th.y - gc.y) + tl.y) * ir, uz = ((th.z - gc.z) + tl.z) * ir;
+  const float r2 = ux * ux + uy * uy + uz * uz;
+  const float i2 = __fdividef(1.f, r2), ri = rsqrt_mufu(r2);
+  const float px = ux * i2, py = uy * i2, wz = uz * i2;
+  float sr = 0.f, si = 0.f;
+  if constexpr (KS < KP) {
+    if (q >= 2 * KS) {
+      float2 CR[KP - KS], CI[KP - KS];
+      series_group<P, KS, KP>(M, wz, i2, ri, q, CR, CI);
+#pragma unroll
+      for (int k = KP - KS - 1; k >= 0; --k) {
+        horner(sr, si, px, py, CR[k].y, CI[k].y);
+        horner(sr, si, px, py, CR[k].x, CI[k].x);
+      }
+    }
+  }
+  float2 CR[KS], CI[KS];
+  series_group<P, 0, KS>(M, wz, i2, ri, q, CR, CI);
+#pragma unroll
+  for (int k = KS - 1; k >= 1; --k) {
+    horner(sr, si, px, py, CR[k].y, CI[k].y);
+    horner(sr, si, px, py, CR[k].x, CI[k].x);
+  }
+  horner(sr, si, px, py, CR[0].y, CI[0].y);
+  // Re(S z) twice, and the real column m = 0
+  return fmaf(2.f, fmaf(sr, px, -si * py), CR[0].x) * ir;
 }
 
 // phi at the target of the far images' expansion (|x| < a)
@@ -617,43 +659,87 @@ __device__ __forceinline__ float l2p_far(const float2* __restrict__ L, float4 th
   return acc * inv_a;
 }
 
-// Direct sum of the records [be.x, be.y) at the lane's target, staged 32 at a time through the
-// warp's shared buffers, with the exact (hi, lo) coordinate difference of inv_hilo (accurate to
-// FP32 rounding at any distance, e.g. a charge next to its own Kelvin image).  checked: the node
-// holds some of the group's own targets, and the source at sorted position `self` is skipped;
+// Direct sum of the records [be.x, be.y) of a node at the lane's target, staged 32 at a time through
+// the warp's shared buffer; two sources per step as packed FP32, side by side in the buffer (a
+// source past the range is far away and has no charge).
+//  EXACT: with the (hi, lo) coordinate difference of inv_hilo (accurate to FP32 rounding at any
+//    distance, e.g. a charge next to its own Kelvin image); checked: the node holds some of the
+//    group's own targets, and the source at sorted position `self` is skipped.
+//  Otherwise, for a node whose radius is at most kRelRadius times its distance from every target:
+//    the difference of the FP32 coordinates relative to the node's centre c.  With
+//    X = |t - c| + rho and d >= |t - c| - rho the rounding of either is at most sqrt(3) u X / d
+//    relative to the distance (u = 2^-24), X / d <= 4: 8e-7, and of either sign.  9 operations for
+//    two pairs instead of 15, half the shared loads and half the staging; nine tenths of the direct pairs
+//    at N = 1e5.
 // kelvin: records beyond rfar2 count as zero.  Each batch's FP32 sum is added to the compensated
 // total (a leaf of a dense cluster holds thousands of sources of similar size and mixed sign).
-__device__ __forceinline__ void p2p(const float4* __restrict__ H, const float4* __restrict__ Lo, int2 be, float4 th,
-                                    float4 tl, int self, bool checked, bool kelvin, float rfar2, float4* sh, float4* sl,
-                                    df& total)
+constexpr float kRelRadius = 0.6f;
+struct P2PShared {
+  float x[32], y[32], z[32], q[32], lx[32], ly[32], lz[32];
+};
+template <bool EXACT>
+__device__ __forceinline__ void p2p(const float4* __restrict__ H, const float4* __restrict__ Lo, int2 be, float4 gc,
+                                    float4 th, float4 tl, int self, bool checked, bool kelvin, float rfar2,
+                                    P2PShared& sh, df& total)
 {
   const int lane = threadIdx.x & 31;
+  // EXACT: the target's hi parts, else its coordinates relative to the centre
+  const float tx = EXACT ? th.x : (th.x - gc.x) + tl.x, ty = EXACT ? th.y : (th.y - gc.y) + tl.y,
+              tz = EXACT ? th.z : (th.z - gc.z) + tl.z;
+  const float2 X = make_float2(tx, tx), Y = make_float2(ty, ty), Z = make_float2(tz, tz);
   for (int j0 = be.x; j0 < be.y; j0 += 32) {
-    float acc = 0.f;  // one batch of 32 sources, folded into the compensated total below
     const int j = j0 + lane;
-    __syncwarp();  // the previous batch has been read
+    float4 h = make_float4(1.0e18f, 0.f, 0.f, 0.f), l = make_float4(0.f, 0.f, 0.f, 0.f);
     if (j < be.y) {
-      float4 h = H[j];
+      h = H[j];
+      l = Lo[j];
       if (kelvin && far_image(h, rfar2)) h.w = 0.f;
-      sh[lane] = h;
-      sl[lane] = Lo[j];
+    }
+    __syncwarp();  // the previous batch has been read
+    // (negated: the differences are sums)
+    sh.x[lane] = EXACT ? -h.x : -((h.x - gc.x) + l.x);
+    sh.y[lane] = EXACT ? -h.y : -((h.y - gc.y) + l.y);
+    sh.z[lane] = EXACT ? -h.z : -((h.z - gc.z) + l.z);
+    sh.q[lane] = h.w;
+    if (EXACT) {
+      sh.lx[lane] = -l.x;
+      sh.ly[lane] = -l.y;
+      sh.lz[lane] = -l.z;
     }
     __syncwarp();
     const int m = min(32, be.y - j0);
-    if (!checked) {
-#pragma unroll 4
-      for (int k = 0; k < m; ++k) {
-        const float4 s = sh[k], u = sl[k];
-        acc = fmaf(s.w, inv_hilo(th.x, th.y, th.z, tl.x, tl.y, tl.z, s.x, s.y, s.z, u.x, u.y, u.z), acc);
+    float2 acc = make_float2(0.f, 0.f);  // one batch of 32 sources
+#pragma unroll 2
+    for (int k = 0; k < m; k += 4) {
+      float4 f[7];
+      f[0] = *reinterpret_cast<const float4*>(&sh.x[k]);
+      f[1] = *reinterpret_cast<const float4*>(&sh.y[k]);
+      f[2] = *reinterpret_cast<const float4*>(&sh.z[k]);
+      f[3] = *reinterpret_cast<const float4*>(&sh.q[k]);
+      if (EXACT) {
+        f[4] = *reinterpret_cast<const float4*>(&sh.lx[k]);
+        f[5] = *reinterpret_cast<const float4*>(&sh.ly[k]);
+        f[6] = *reinterpret_cast<const float4*>(&sh.lz[k]);
       }
-    } else {
-      for (int k = 0; k < m; ++k) {
-        const float4 s = sh[k], u = sl[k];
-        const float v = s.w * inv_hilo(th.x, th.y, th.z, tl.x, tl.y, tl.z, s.x, s.y, s.z, u.x, u.y, u.z);
-        acc += (j0 + k == self) ? 0.f : v;
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        auto two = [&](int i) { return p ? make_float2(f[i].z, f[i].w) : make_float2(f[i].x, f[i].y); };
+        float2 ex = __fadd2_rn(X, two(0)), ey = __fadd2_rn(Y, two(1)), ez = __fadd2_rn(Z, two(2));
+        if (EXACT) {
+          ex = __fadd2_rn(__fadd2_rn(make_float2(tl.x, tl.x), two(4)), ex);
+          ey = __fadd2_rn(__fadd2_rn(make_float2(tl.y, tl.y), two(5)), ey);
+          ez = __fadd2_rn(__fadd2_rn(make_float2(tl.z, tl.z), two(6)), ez);
+        }
+        const float2 r2 = __ffma2_rn(ez, ez, __ffma2_rn(ey, ey, __fmul2_rn(ex, ex)));
+        float2 inv = make_float2(rsqrt_mufu(r2.x), rsqrt_mufu(r2.y));
+        if (EXACT && checked) {  // the target itself
+          if (j0 + k + 2 * p == self) inv.x = 0.f;
+          if (j0 + k + 2 * p + 1 == self) inv.y = 0.f;
+        }
+        acc = __ffma2_rn(two(3), inv, acc);
       }
     }
-    total = total + two_sum(acc, 0.f);
+    total = total + two_sum(acc.x, acc.y);
   }
 }
 
@@ -663,9 +749,9 @@ __device__ __forceinline__ void p2p(const float4* __restrict__ H, const float4* 
 // written to the item's own partial row (chunk tr kTreeRootSplit + rs).
 template <int P>
 __device__ __forceinline__ void eval_group(const TreeView& t, float2* __restrict__ part, int grp, int tr, int rs,
-                                           int* stk, int2* sbe, float4* sgc, float4* sh, float4* sl, float2* smom)
+                                           int* stk, int2* sbe, float4* sgc, P2PShared& sp2, float4* smom)
 {
-  constexpr int NM = tree_nm(P);
+  constexpr int NQ = tree_nq(P);
   const int lane = threadIdx.x & 31;
   const SysDev& S = t.sys[0];
   const int n = S.n;
@@ -681,7 +767,7 @@ __device__ __forceinline__ void eval_group(const TreeView& t, float2* __restrict
     const float4* __restrict__ H = t.hi + S.src + (long long)tr * n;
     const float4* __restrict__ Lo = t.lo + S.src + (long long)tr * n;
     const float4* __restrict__ G = t.geo + (long long)tr * nodes;
-    const float2* __restrict__ MM = t.mom + (long long)tr * nodes * NM;
+    const float4* __restrict__ MM = t.mom + (long long)tr * nodes * NQ;
     const int self = tr == 0 ? i : -1;
     __syncwarp();
     constexpr int RS = R / kTreeRootSplit;
@@ -716,38 +802,39 @@ __device__ __forceinline__ void eval_group(const TreeView& t, float2* __restrict
       const float4 gc = sgc[sp];
       __syncwarp();  // every lane has read the entry before a push overwrites it
       const int l = e >> 26, c = e & ((1 << 26) - 1);
-      const long long g = tree_node_index(l, c);
+      const int g = (int)tree_node_index(l, 0) + c;  // (levels to 7: below 2^22)
       // the node is far when its series converges with ratio rho / |t - c| <= theta at every
       // target of the group (each lane tests its own target; a margin covers the lo parts)
       const float dx = th.x - gc.x, dy = th.y - gc.y, dz = th.z - gc.z;
       const float rm = gc.w + margin;
-      const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-      const bool far = __all_sync(0xffffffffu, rm * rm <= theta2 * d2);
+      // (the nearest target decides: one reduction serves the three tests of the node)
+      const float d2 = __uint_as_float(
+          __reduce_min_sync(0xffffffffu, __float_as_uint(fmaf(dz, dz, fmaf(dy, dy, dx * dx)))));
+      const bool far = rm * rm <= theta2 * d2;
       if (far && be.y - be.x >= t.cmin) {
         // the order whose truncation at the group's largest ratio rho/|t - c| stays within a tenth
-        // of the order-P bound at theta: (q + 1) log(ratio) <= log(0.1 theta^(P+1))
+        // of the order-P bound at theta: (q + 1) log(ratio) <= log(0.1 theta^(P+1)); order 16 keeps
+        // every node at its order
+        int q = P;
         if constexpr (P <= 12) {
-          const float r2max = warp_max(rm * rm / d2);
-          const int q = min(P, max(2, (int)ceilf(t.log_eps / (0.5f * __logf(r2max))) - 1));
-          // the node's moments staged in shared memory by one coalesced warp load
-          const float2* src = MM + g * NM;
-          for (int i = lane; i < NM; i += 32) {
-            const float2 v = __ldg(src + i);
-            smom[i] = make_float2(v.x, -v.y);  // (re, -im): the series' dot product as FFMA2
-          }
-          __syncwarp();
-          acc = acc + two_sum(m2p_rows<P>(smom, gc, th, tl, q), 0.f);
-          __syncwarp();
-        } else {
-          // (two rows of order 16 do not fit the registers: every node at order P, by columns)
-          acc = acc + two_sum(m2p<P, P>(MM + g * NM, gc, th, tl), 0.f);
+          q = min(P, max(2, (int)ceilf(__fdividef(t.log_eps, 0.5f * __logf(__fdividef(rm * rm, d2)))) - 1));
         }
+        // the node's moments staged in shared memory by coalesced warp loads
+        const float4* src = MM + (size_t)g * NQ;
+        for (int i = lane; i < NQ; i += 32) smom[i] = __ldg(src + i);
+        __syncwarp();
+        acc = acc + two_sum(m2p<P>(smom, gc, th, tl, q), 0.f);
+        __syncwarp();
       } else if (far || l == t.L) {
-        const bool checked = tr == 0 && be.x < grp * 32 + 32 && be.y > grp * 32;
-        p2p(H, Lo, be, th, tl, self, checked, tr == 1, t.rfar2, sh, sl, acc);
+        if (rm * rm <= kRelRadius * kRelRadius * d2) {
+          p2p<false>(H, Lo, be, gc, th, tl, -1, false, tr == 1, t.rfar2, sp2, acc);
+        } else {
+          const bool checked = tr == 0 && be.x < grp * 32 + 32 && be.y > grp * 32;
+          p2p<true>(H, Lo, be, gc, th, tl, self, checked, tr == 1, t.rfar2, sp2, acc);
+        }
       } else {
         // open: the children with sources, the lowest cell on top
-        const long long gch = tree_node_index(l + 1, 8LL * c);
+        const int gch = 8 * g + 1;  // the first child: 8 ((8^l - 1)/7 + c) + 1
         int2 cb = make_int2(0, 0);
         float4 cg = make_float4(0.f, 0.f, 0.f, -1.f);
         if (lane < 8) {
@@ -774,12 +861,12 @@ template <int P>
 __global__ __launch_bounds__(32 * kTreeEvalWarps, kTreeEvalMinBlocks) void k_tree_eval(TreeView t,
                                                                                        float2* __restrict__ part)
 {
-  constexpr int NM = tree_nm(P);
+  constexpr int NQ = tree_nq(P);
   __shared__ int s_stack[kTreeEvalWarps][kTreeStack];
   __shared__ int2 s_sbe[kTreeEvalWarps][kTreeStack];
   __shared__ float4 s_sgc[kTreeEvalWarps][kTreeStack];
-  __shared__ float2 s_mom[kTreeEvalWarps][NM];
-  __shared__ float4 s_h[kTreeEvalWarps][32], s_l[kTreeEvalWarps][32];
+  __shared__ float4 s_mom[kTreeEvalWarps][NQ];
+  __shared__ __align__(16) P2PShared s_p2p[kTreeEvalWarps];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const SysDev& S = t.sys[0];
   const int n = S.n;
@@ -789,7 +876,7 @@ __global__ __launch_bounds__(32 * kTreeEvalWarps, kTreeEvalMinBlocks) void k_tre
   // cost of an item varies with its distance from the interface and from the centre)
   for (int it = blockIdx.x * kTreeEvalWarps + w; it < items;) {
     const int r = it % IPG;
-    eval_group<P>(t, part, it / IPG, r & 1, r >> 1, s_stack[w], s_sbe[w], s_sgc[w], s_h[w], s_l[w], s_mom[w]);
+    eval_group<P>(t, part, it / IPG, r & 1, r >> 1, s_stack[w], s_sbe[w], s_sgc[w], s_p2p[w], s_mom[w]);
     int nx = 0;
     if (lane == 0) nx = workers + (int)atomicAdd(t.ctr + 1, 1u);
     it = __shfl_sync(0xffffffffu, nx, 0);
@@ -813,7 +900,7 @@ static void build_p(const TreeView& t, int n, cudaStream_t st)
   k_tree_leaf<P><<<(unsigned)((leaves + kLeafWarps - 1) / kLeafWarps), 32 * kLeafWarps, 0, st>>>(t);
   for (int l = t.L - 1; l >= kTreeTop; --l) {
     const long long cells = 1LL << (3 * l);
-    k_tree_up<P><<<(unsigned)((cells + kUpWarps - 1) / kUpWarps), 32 * kUpWarps, 0, st>>>(t, l);
+    k_tree_up<P><<<dim3((unsigned)cells, 2), 32 * up_warps<P>(), 0, st>>>(t, l);
   }
 }
 

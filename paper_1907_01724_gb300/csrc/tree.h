@@ -20,13 +20,14 @@ constexpr int kTreeMaxLevel = 7;  // finest node level supported
 constexpr int kFarOrder = 24;     // order of the origin-centred expansion of the far images
 constexpr float kFarImageRel = 2.0f;  // Kelvin images beyond this multiple of a: far images
 constexpr int kTreeEvalWarps = 4;     // warps (persistent target-group workers) per k_tree_eval block
-constexpr int kTreeEvalMinBlocks = 7; // resident k_tree_eval blocks per SM the kernel is built for
+constexpr int kTreeEvalMinBlocks = 6; // resident k_tree_eval blocks per SM the kernel is built for
 constexpr int kTreeStack = 128;       // traversal stack entries per warp
 constexpr int kFarBlocks = 512;       // blocks of k_tree_far
 
 __host__ __device__ constexpr long long tree_node_index(int l, long long c) { return ((1LL << (3 * l)) - 1) / 7 + c; }
 __host__ __device__ constexpr long long tree_node_count(int L) { return ((1LL << (3 * (L + 1))) - 1) / 7; }
 __host__ __device__ constexpr int tree_nm(int P) { return (P + 1) * (P + 2) / 2; }  // complex moments n <= P, 0 <= m <= n
+__host__ __device__ constexpr int tree_nq(int P) { return (P / 2 + 1) * (P / 2 + 1); }  // float4 entries of a node's moments
 
 // Everything the tree kernels read and write (device pointers into the engine's workspace;
 // one system).
@@ -39,7 +40,7 @@ struct TreeView {
   int2* node;                // [nodes]: record range [begin, end) of every node
   float4* geo;               // [2][nodes]: centre and radius of the real / Kelvin sources (radius < 0: none)
   float4* box;               // [2][nodes][2]: bounding box (min, max) of the same
-  float2* mom;               // [2][nodes][nm]: multipole moments about the centre, in units of the radius
+  float4* mom;               // [2][nodes][nq]: multipole moments about the centre, in units of the radius
   float2* farp;              // [kFarBlocks][tree_nm(kFarOrder)]: block partials of the far-image expansion
   float2* farL;              // [tree_nm(kFarOrder)]: the far-image expansion
   unsigned int* ctr;         // [0]: completion counter of k_tree_far, [1]: k_tree_eval's work counter

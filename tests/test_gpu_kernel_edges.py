@@ -38,3 +38,21 @@ def test_default_tile_configurations(n):
     api.hsma_build_sources(h, xyz, q)
     assert np.linalg.norm(api.hsma_potential(h) - ref) <= 1e-6 * np.linalg.norm(ref)
     assert np.linalg.norm(api.hsma_field(h) - E) <= 1e-6 * np.linalg.norm(E)
+
+
+@pytest.mark.parametrize("order", [8, 12, 16])
+@pytest.mark.parametrize("n", [2, 5, 36, 513, 4097])
+def test_tree_at_batch_edges(n, order):
+    """The far-field tree where its batches of 32 and steps of 4 sources end, with charges at the
+    centre's images (far), next to the interface (their own images: the exact direct sum) and in one
+    dense cell, against the FP64 path's direct sum (order 8 at theta 0.35; 1e-6 norm-wise)."""
+    rng = np.random.default_rng(190810 + n)
+    k = n // 3
+    xyz = np.concatenate([inputs.shell(rng, k, 1.0, 1e-3), inputs.uniform_ball(rng, k, 0.3),
+                          np.array([0.3, 0.2, -0.4]) + inputs.uniform_ball(rng, n - 2 * k, 0.02)])
+    s = inputs.System(1.0, 2.0, 80.0, 1.5, 12, 400, xyz, rng.choice([-1.0, 1.0], n))
+    ref = api.solve(s, precision=api.HSMA_FP64).phi
+    h = api.hsma_create(s.a, s.eps1, s.eps2, s.kappa, api.hsma_default_params(p=s.p, M=s.M))
+    api.hsma_set_far_field(h, 0.35 if order == 8 else 0.5, order)
+    api.hsma_build_sources(h, s.xyz, s.q)
+    assert np.linalg.norm(api.hsma_potential(h) - ref) <= 1e-6 * np.linalg.norm(ref)
