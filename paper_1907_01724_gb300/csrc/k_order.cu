@@ -93,7 +93,13 @@ __global__ __launch_bounds__(kKeyThreads) void k_order_keys(const SysDev* __rest
 // they are at most smem_n (the launch's dynamic shared memory, sized by the engine), else in the
 // scratch buffer scr (2 ints per charge of the system: input indices, then cells).  done[s]
 // counts the system's blocks that have read the histogram; the last one zeroes both.
+//
+// With a finer key (the far-field tree) a cell holds hundreds of charges, and ranking each against
+// its whole cell took most of the kernel (1.37 ms at N = 1e6).  The block's slots are then binned once
+// more by the key's next bits (as many as give at most kSortSub bins), through the scratch buffer, and
+// ranked inside their bin: 0.28 ms.
 constexpr int kSortThreads = 512;
+constexpr int kSortSub = 4096;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortBatch = 8;  // keys in flight per thread
 static_assert(kOrderCells % kSortThreads == 0, "cells split evenly over the sort block");
@@ -105,6 +111,7 @@ __global__ __launch_bounds__(kSortThreads) void k_order_sort(const SysDev* __res
                                                              int* __restrict__ perm, int smem_n)
 {
   __shared__ int s_cell[kOrderCells];
+  __shared__ int s_sub[kSortSub];
   __shared__ int s_wsum[kSortWarps];
   __shared__ int s_last;
   extern __shared__ int s_slot[];
@@ -192,6 +199,60 @@ __global__ __launch_bounds__(kSortThreads) void k_order_sort(const SysDev* __res
     }
   }
   __syncthreads();
+
+  if (ksh > 0 && m <= smem_n) {
+    int sub = 0;  // bits of the key below its cell that choose the bin
+    while (sub < ksh && ((k1 - k0) << (sub + 1)) <= kSortSub) ++sub;
+    const int sh = ksh - sub, first = k0 << sub;
+    for (int b = tid; b < kSortSub; b += kSortThreads) s_sub[b] = 0;
+    __syncthreads();
+    for (int a = tid; a < m; a += kSortThreads) atomicAdd(&s_sub[(skey[a] >> sh) - first], 1);
+    __syncthreads();
+    // exclusive scan of the bins
+    constexpr int pb = kSortSub / kSortThreads;
+    int c[pb], tot = 0;
+#pragma unroll
+    for (int j = 0; j < pb; ++j) {
+      c[j] = s_sub[tid * pb + j];
+      tot += c[j];
+    }
+    int inc = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
+    }
+    if (lane == 31) s_wsum[warp] = inc;
+    __syncthreads();
+    int at = inc - tot;
+    for (int w = 0; w < warp; ++w) at += s_wsum[w];
+#pragma unroll
+    for (int j = 0; j < pb; ++j) {
+      s_sub[tid * pb + j] = at;
+      at += c[j];
+    }
+    __syncthreads();
+    int* slot2 = scr + 2 * c0 + P0;
+    int* skey2 = scr + 2 * c0 + n + P0;
+    for (int a = tid; a < m; a += kSortThreads) {
+      const int p = atomicAdd(&s_sub[(skey[a] >> sh) - first], 1);
+      slot2[p] = slot[a];
+      skey2[p] = skey[a];
+    }
+    __syncthreads();
+    // (s_sub[b] is now the end of bin b; the bins follow one another)
+    for (int a = tid; a < m; a += kSortThreads) {
+      const int v = slot2[a], kf = skey2[a], b = (kf >> sh) - first;
+      const int b0 = b > 0 ? s_sub[b - 1] : 0, e = s_sub[b];
+      int p = b0;
+      for (int x = b0; x < e; ++x) {
+        const int kb = skey2[x];
+        p += kb < kf || (kb == kf && slot2[x] < v);
+      }
+      perm[c0 + P0 + p] = v;
+    }
+    return;
+  }
 
   // slot a of cell k (which spans [end of cell k - 1, end of cell k), the first from P0) goes to
   // the cell's start plus the number of the cell's charges before it: the input indices below

@@ -109,6 +109,25 @@ __device__ __forceinline__ float warp_sum(float v)
   return v;
 }
 
+// Sums of N <= 32 values over the warp's lanes, transposed: lane l returns the sum of value l
+// (garbage for l >= N).  31 shuffles for 32 sums, where a butterfly for each takes 160; the same
+// pairs are added, so the sums are those of warp_sum to the bit.
+template <int N>
+__device__ __forceinline__ float warp_sums(float (&v)[N], int lane)
+{
+  static_assert(N == 32, "one value per lane");
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < o; ++k) {
+      const float keep = up ? v[o + k] : v[k], give = up ? v[k] : v[o + k];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  return v[0];
+}
+
 // ---------------------------------------------------------------------------------------
 // Record ranges: sorted position i starts node (l, c) if the previous record's key prefix
 // differs, and ends it if the next one's does.  node[] is zeroed before (empty nodes keep 0, 0).
@@ -132,7 +151,10 @@ __global__ __launch_bounds__(256) void k_tree_marks(TreeView t)
 }
 
 // ---------------------------------------------------------------------------------------
-// Leaves: geometry and moments of both trees, a warp per level-L node.
+// Leaves: geometry and moments, a warp per (level-L node, tree).  Columns m and P - m together have
+// P + 2 coefficients whatever m, 2 (P + 2) sums of one transposed reduction (two of them for order
+// 16), and the records are read once per pair of columns: 36 and 216 us at N = 1e5 and 1e6, 98 and
+// 555 with both trees in one warp and a butterfly per sum.
 constexpr int kLeafWarps = 4;
 template <int P>
 __global__ __launch_bounds__(32 * kLeafWarps) void k_tree_leaf(TreeView t)
@@ -147,94 +169,121 @@ __global__ __launch_bounds__(32 * kLeafWarps) void k_tree_leaf(TreeView t)
   const long long g = tree_node_index(t.L, c);
   const int2 be = t.node[g];
   const float a = 1.f / t.inv_a;
-  for (int tr = 0; tr < 2; ++tr) {
-    const float4* __restrict__ H = t.hi + S.src + (long long)tr * n;
-    const float4* __restrict__ Lo = t.lo + S.src + (long long)tr * n;
-    float mn0 = 3.0e38f, mn1 = 3.0e38f, mn2 = 3.0e38f, mx0 = -3.0e38f, mx1 = -3.0e38f, mx2 = -3.0e38f;
-    for (int j = be.x + lane; j < be.y; j += 32) {
-      const float4 h = H[j];
-      if (tr == 1 && far_image(h, t.rfar2)) continue;
-      mn0 = fminf(mn0, h.x);
-      mn1 = fminf(mn1, h.y);
-      mn2 = fminf(mn2, h.z);
-      mx0 = fmaxf(mx0, h.x);
-      mx1 = fmaxf(mx1, h.y);
-      mx2 = fmaxf(mx2, h.z);
-    }
-    mn0 = warp_min(mn0);
-    mn1 = warp_min(mn1);
-    mn2 = warp_min(mn2);
-    mx0 = warp_max(mx0);
-    mx1 = warp_max(mx1);
-    mx2 = warp_max(mx2);
-    float4* geo = t.geo + (long long)tr * nodes + g;
-    float4* bx = t.box + 2 * ((long long)tr * nodes + g);
-    float4* M = t.mom + ((long long)tr * nodes + g) * NQ;
-    if (!(mn0 <= mx0)) {
-      if (lane == 0) {
-        *geo = make_float4(0.f, 0.f, 0.f, -1.f);
-        bx[0] = make_float4(3.0e38f, 3.0e38f, 3.0e38f, 0.f);
-        bx[1] = make_float4(-3.0e38f, -3.0e38f, -3.0e38f, 0.f);
-      }
-      for (int k = lane; k < NQ; k += 32) M[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-      continue;
-    }
-    const float cx = 0.5f * (mn0 + mx0), cy = 0.5f * (mn1 + mx1), cz = 0.5f * (mn2 + mx2);
-    float r2max = 0.f;
-    for (int j = be.x + lane; j < be.y; j += 32) {
-      const float4 h = H[j];
-      if (tr == 1 && far_image(h, t.rfar2)) continue;
-      const float dx = h.x - cx, dy = h.y - cy, dz = h.z - cz;
-      r2max = fmaxf(r2max, dx * dx + dy * dy + dz * dz);
-    }
-    // (a margin for the rounding of the hi coordinates and of the distance)
-    const float rho = sqrtf(warp_max(r2max)) * 1.000001f + 2e-7f * a + 1e-6f * a;
+  const int tr = blockIdx.y;
+  const float4* __restrict__ H = t.hi + S.src + (long long)tr * n;
+  const float4* __restrict__ Lo = t.lo + S.src + (long long)tr * n;
+  float mn0 = 3.0e38f, mn1 = 3.0e38f, mn2 = 3.0e38f, mx0 = -3.0e38f, mx1 = -3.0e38f, mx2 = -3.0e38f;
+  for (int j = be.x + lane; j < be.y; j += 32) {
+    const float4 h = H[j];
+    if (tr == 1 && far_image(h, t.rfar2)) continue;
+    mn0 = fminf(mn0, h.x);
+    mn1 = fminf(mn1, h.y);
+    mn2 = fminf(mn2, h.z);
+    mx0 = fmaxf(mx0, h.x);
+    mx1 = fmaxf(mx1, h.y);
+    mx2 = fmaxf(mx2, h.z);
+  }
+  mn0 = warp_min(mn0);
+  mn1 = warp_min(mn1);
+  mn2 = warp_min(mn2);
+  mx0 = warp_max(mx0);
+  mx1 = warp_max(mx1);
+  mx2 = warp_max(mx2);
+  float4* geo = t.geo + (long long)tr * nodes + g;
+  float4* bx = t.box + 2 * ((long long)tr * nodes + g);
+  float4* M = t.mom + ((long long)tr * nodes + g) * NQ;
+  if (!(mn0 <= mx0)) {
     if (lane == 0) {
-      *geo = make_float4(cx, cy, cz, rho);
-      bx[0] = make_float4(mn0, mn1, mn2, 0.f);
-      bx[1] = make_float4(mx0, mx1, mx2, 0.f);
+      *geo = make_float4(0.f, 0.f, 0.f, -1.f);
+      bx[0] = make_float4(3.0e38f, 3.0e38f, 3.0e38f, 0.f);
+      bx[1] = make_float4(-3.0e38f, -3.0e38f, -3.0e38f, 0.f);
     }
-    const float ir = inv_unit(rho);
+    for (int k = lane; k < NQ; k += 32) M[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    return;
+  }
+  const float cx = 0.5f * (mn0 + mx0), cy = 0.5f * (mn1 + mx1), cz = 0.5f * (mn2 + mx2);
+  float r2max = 0.f;
+  for (int j = be.x + lane; j < be.y; j += 32) {
+    const float4 h = H[j];
+    if (tr == 1 && far_image(h, t.rfar2)) continue;
+    const float dx = h.x - cx, dy = h.y - cy, dz = h.z - cz;
+    r2max = fmaxf(r2max, dx * dx + dy * dy + dz * dz);
+  }
+  // (a margin for the rounding of the hi coordinates and of the distance)
+  const float rho = sqrtf(warp_max(r2max)) * 1.000001f + 2e-7f * a + 1e-6f * a;
+  if (lane == 0) {
+    *geo = make_float4(cx, cy, cz, rho);
+    bx[0] = make_float4(mn0, mn1, mn2, 0.f);
+    bx[1] = make_float4(mx0, mx1, mx2, 0.f);
+  }
+  const float ir = inv_unit(rho);
 #pragma unroll
-    for (int m = 0; m <= P; ++m) {
-      float cr[P + 1], ci[P + 1];
+  for (int m0 = 0; 2 * m0 <= P; ++m0) {
+    constexpr int NC = P + 2;
+    float cr[NC], ci[NC];  // column m0 (n = m0..P), then column P - m0
 #pragma unroll
-      for (int k = 0; k <= P - m; ++k) cr[k] = ci[k] = 0.f;
-      for (int j = be.x + lane; j < be.y; j += 32) {
-        const float4 h = H[j];
-        if (tr == 1 && far_image(h, t.rfar2)) continue;
-        const float4 l = Lo[j];
-        const float vx = ((h.x - cx) + l.x) * ir, vy = ((h.y - cy) + l.y) * ir, vz = ((h.z - cz) + l.z) * ir;
-        const float r2 = vx * vx + vy * vy + vz * vz;
-        float dr = h.w, di = 0.f;  // Q R_m^m
+    for (int k = 0; k < NC; ++k) cr[k] = ci[k] = 0.f;
+    for (int j = be.x + lane; j < be.y; j += 32) {
+      const float4 h = H[j];
+      if (tr == 1 && far_image(h, t.rfar2)) continue;
+      const float4 l = Lo[j];
+      const float vx = ((h.x - cx) + l.x) * ir, vy = ((h.y - cy) + l.y) * ir, vz = ((h.z - cz) + l.z) * ir;
+      const float r2 = vx * vx + vy * vy + vz * vz;
+      float dr = h.w, di = 0.f;  // Q R_m^m
 #pragma unroll
-        for (int k = 1; k <= m; ++k) {
+      for (int half = 0; half < 2; ++half) {
+        const int m = half ? P - m0 : m0;
+        if (half && 2 * m0 == P) break;
+#pragma unroll
+        for (int k = half ? m0 + 1 : 1; k <= m; ++k) {
           const float s = 0.5f / (float)k;
           const float nr = (dr * vx - di * vy) * s;
           di = (dr * vy + di * vx) * s;
           dr = nr;
         }
+        const int at = half ? P - m0 + 1 : 0;
         float p0r = 0.f, p0i = 0.f, p1r = dr, p1i = di;
-        cr[0] += p1r;
-        ci[0] -= p1i;
+        cr[at] += p1r;
+        ci[at] -= p1i;
 #pragma unroll
         for (int nn = m + 1; nn <= P; ++nn) {
           const float A = (float)(2 * nn - 1) * vz;
           const float inv = 1.f / (float)(nn * nn - m * m);
           const float qr = (A * p1r - r2 * p0r) * inv, qi = (A * p1i - r2 * p0i) * inv;
-          cr[nn - m] += qr;
-          ci[nn - m] -= qi;
+          cr[at + nn - m] += qr;
+          ci[at + nn - m] -= qi;
           p0r = p1r;
           p0i = p1i;
           p1r = qr;
           p1i = qi;
         }
       }
+    }
+    // lane k: the real parts of coefficient k, lane 16 + k (order 16: another reduction) the imaginary
+    float sr, si;
+    if constexpr (NC <= 16) {
+      float v[32];
 #pragma unroll
-      for (int k = 0; k <= P - m; ++k) {
-        const float sr = warp_sum(cr[k]), si = warp_sum(ci[k]);
-        if (lane == 0) put_moment(M, P, m + k, m, sr, si);
+      for (int k = 0; k < 16; ++k) {
+        v[k] = k < NC ? cr[k] : 0.f;
+        v[16 + k] = k < NC ? ci[k] : 0.f;
       }
+      sr = warp_sums(v, lane);
+      si = __shfl_xor_sync(0xffffffffu, sr, 16);
+    } else {
+      float v[32], u[32];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) {
+        v[k] = k < NC ? cr[k] : 0.f;
+        u[k] = k < NC ? ci[k] : 0.f;
+      }
+      sr = warp_sums(v, lane);
+      si = warp_sums(u, lane);
+    }
+    const int nc0 = P - m0 + 1;
+    if (lane < (2 * m0 == P ? nc0 : NC)) {
+      const int m = lane < nc0 ? m0 : P - m0, n_ = lane < nc0 ? m0 + lane : P - m0 + lane - nc0;
+      put_moment(M, P, n_, m, sr, si);
     }
   }
 }
@@ -427,25 +476,27 @@ __global__ __launch_bounds__(32 * (P > 12 ? 4 : 8)) void k_tree_up(TreeView t, i
 }
 
 // ---------------------------------------------------------------------------------------
-// Far images: L_n^m = sum Q conj(I_n^m(y/a)) over Kelvin records beyond kFarImageRel a.
+// Far images: L_n^m = sum Q conj(I_n^m(y/a)) over Kelvin records beyond kFarImageRel a.  A block takes
+// batches of 32 records dealt out over the grid (far images are runs of the order: a block with its
+// own run of records had all of the work or none), its warps the columns m = w, w + 8, ... of a batch
+// (the latency of all 325 sums in one warp was the kernel: 87 and 373 us at N = 1e5 and 1e6; 62 and 213 so).
 constexpr int kFarWarps = 8;
 constexpr int kFarNM = tree_nm(kFarOrder);
 __global__ __launch_bounds__(32 * kFarWarps) void k_tree_far(TreeView t)
 {
+  __shared__ float2 sum[kFarNM];  // the block's sums (a column belongs to one warp)
   __shared__ float2 acc[kFarWarps][kFarNM];
   __shared__ bool last;
   const SysDev& S = t.sys[0];
   const int n = S.n;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < kFarWarps * kFarNM; i += blockDim.x) (&acc[0][0])[i] = make_float2(0.f, 0.f);
+  for (int i = threadIdx.x; i < kFarNM; i += blockDim.x) sum[i] = make_float2(0.f, 0.f);
   __syncthreads();
-  const int per = ((n + kFarBlocks - 1) / kFarBlocks + 31) / 32 * 32;
-  const int r0 = blockIdx.x * per, r1 = min(n, r0 + per);
-  for (int j0 = r0 + 32 * w; j0 < r1; j0 += 32 * kFarWarps) {
+  for (int j0 = 32 * blockIdx.x; j0 < n; j0 += 32 * gridDim.x) {
     const int j = j0 + lane;
     float4 h = make_float4(0.f, 0.f, 0.f, 0.f), lo = h;
     bool far = false;
-    if (j < r1) {
+    if (j < n) {
       h = t.hi[S.src + n + j];
       far = far_image(h, t.rfar2);
       if (far) lo = t.lo[S.src + n + j];
@@ -466,6 +517,7 @@ __global__ __launch_bounds__(32 * kFarWarps) void k_tree_far(TreeView t)
         di = (dr * uy + di * ux) * f;
         dr = nr;
       }
+      if (m % kFarWarps != w) continue;  // whole warps
       float cr[kFarOrder + 1], ci[kFarOrder + 1];
       float p0r = 0.f, p0i = 0.f, p1r = dr, p1i = di;
       cr[0] = p1r;
@@ -481,16 +533,38 @@ __global__ __launch_bounds__(32 * kFarWarps) void k_tree_far(TreeView t)
         p1r = qr;
         p1i = qi;
       }
+      float v[32], u[32];
 #pragma unroll
-      for (int k = 0; k <= kFarOrder - m; ++k) {
-        const float sr = warp_sum(cr[k]), si = warp_sum(ci[k]);
-        if (lane == 0) {
-          float2& a = acc[w][tree_col(kFarOrder, m) + k];
-          a.x += sr;
-          a.y += si;
-        }
+      for (int k = 0; k < 32; ++k) {
+        v[k] = k <= kFarOrder - m ? cr[k] : 0.f;
+        u[k] = k <= kFarOrder - m ? ci[k] : 0.f;
+      }
+      const float sr = warp_sums(v, lane), si = warp_sums(u, lane);
+      if (lane <= kFarOrder - m) {
+        float2& a = sum[tree_col(kFarOrder, m) + lane];
+        a.x += sr;
+        a.y += si;
       }
     }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < kFarNM; i += blockDim.x) t.farp[(long long)blockIdx.x * kFarNM + i] = sum[i];
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(t.ctr, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  // warp w adds blocks w, w + kFarWarps, ..., then the warps' sums in order
+  for (int i = lane; i < kFarNM; i += 32) {
+    float2 s = make_float2(0.f, 0.f);
+#pragma unroll 8
+    for (int b = w; b < (int)gridDim.x; b += kFarWarps) {
+      const float2 v = __ldcg(t.farp + (long long)b * kFarNM + i);
+      s.x += v.x;
+      s.y += v.y;
+    }
+    acc[w][i] = s;
   }
   __syncthreads();
   for (int i = threadIdx.x; i < kFarNM; i += blockDim.x) {
@@ -499,21 +573,6 @@ __global__ __launch_bounds__(32 * kFarWarps) void k_tree_far(TreeView t)
     for (int q = 0; q < kFarWarps; ++q) {
       s.x += acc[q][i].x;
       s.y += acc[q][i].y;
-    }
-    t.farp[(long long)blockIdx.x * kFarNM + i] = s;
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(t.ctr, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  for (int i = threadIdx.x; i < kFarNM; i += blockDim.x) {
-    float2 s = make_float2(0.f, 0.f);
-    for (int b = 0; b < (int)gridDim.x; ++b) {
-      const float2 v = __ldcg(t.farp + (long long)b * kFarNM + i);
-      s.x += v.x;
-      s.y += v.y;
     }
     t.farL[i] = s;
   }
@@ -897,7 +956,7 @@ template <int P>
 static void build_p(const TreeView& t, int n, cudaStream_t st)
 {
   const long long leaves = 1LL << (3 * t.L);
-  k_tree_leaf<P><<<(unsigned)((leaves + kLeafWarps - 1) / kLeafWarps), 32 * kLeafWarps, 0, st>>>(t);
+  k_tree_leaf<P><<<dim3((unsigned)((leaves + kLeafWarps - 1) / kLeafWarps), 2), 32 * kLeafWarps, 0, st>>>(t);
   for (int l = t.L - 1; l >= kTreeTop; --l) {
     const long long cells = 1LL << (3 * l);
     k_tree_up<P><<<dim3((unsigned)cells, 2), 32 * up_warps<P>(), 0, st>>>(t, l);
