@@ -555,7 +555,7 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_o
   {
     int per_req = 1;
     for (const auto& d : L.sd)
-      per_req = std::max(per_req, (d.n + kDeltaBlock - 1) / kDeltaBlock + (d.M + kDeltaBlock - 1) / kDeltaBlock);
+      per_req = std::max(per_req, (d.n + kDeltaRows - 1) / kDeltaRows + (d.M + kDeltaBlock - 1) / kDeltaBlock);
     L.max_req = std::max(1, max_requests);
     L.ditem_cap = L.max_req * per_req;
     int surf_blocks = 1;
@@ -1968,7 +1968,7 @@ int Engine::delta_batch(const std::vector<DeltaReq>& reqs, double* de_host)
   for (size_t r = 0; r < reqs.size(); ++r) {
     const SysDev& d = L.sd[reqs[r].sys];
     ranges[r].x = (int)items.size();
-    for (int b = 0; b < (d.n + kDeltaBlock - 1) / kDeltaBlock; ++b) items.push_back(make_int4((int)r, 0, b, 0));
+    for (int b = 0; b < (d.n + kDeltaRows - 1) / kDeltaRows; ++b) items.push_back(make_int4((int)r, 0, b, 0));
     for (int b = 0; b < (d.M + kDeltaBlock - 1) / kDeltaBlock; ++b) items.push_back(make_int4((int)r, 1, b, 0));
     ranges[r].y = (int)items.size() - ranges[r].x;
   }

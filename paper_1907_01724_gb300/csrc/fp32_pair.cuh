@@ -1,5 +1,5 @@
-// Device helpers of the FP32 pair sums (pair, field, move and allocation-free kernels): the MUFU
-// reciprocal square root, cp.async staging, and the (hi, lo) FP32 split of an FP64 value.
+// Device helpers of the pair sums (pair, field, move and allocation-free kernels): the MUFU
+// reciprocal square root (FP32, and refined to FP64), cp.async staging, and the (hi, lo) FP32 split of an FP64 value.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -13,6 +13,20 @@ __device__ __forceinline__ float rsqrt_mufu(float x)
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+
+// 1/sqrt(x): the approximate reciprocal root (relative error below 2^-19), then, with e = 1 - x y^2,
+// y + y e (1/2 + 3/8 e) (the next term, 5/16 e^3, is below 2^-56).  Arguments whose exponent leaves
+// no room for the step (zero, subnormal, near overflow, not finite) take the square root and the
+// division.
+__device__ __forceinline__ double rsqrt_f64(double x)
+{
+  const unsigned int top = (unsigned int)__double2hiint(x) >> 20;  // sign and exponent
+  if (top - 0x040u > 0x780u - 0x040u) return 1.0 / sqrt(x);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 // 16-byte asynchronous global -> shared copy (both addresses 16-byte aligned), its commit group

@@ -350,7 +350,8 @@ struct DeltaReq {
   int k;
   double x, y, z;
 };
-constexpr int kDeltaBlock = 256;  // rows / surface points per delta work item
+constexpr int kDeltaBlock = 256;  // surface points per delta work item, threads of a block
+constexpr int kDeltaRows = 1024;  // rows per delta work item
 void init_delta_kernels();
 void launch_surface_potentials(const SysDev* sys, const int2* items, int nitems, const double* xyz, const double* q,
                                const dbl4* surfx, double2* vsurf, cudaStream_t st);

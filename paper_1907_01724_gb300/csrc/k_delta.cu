@@ -74,24 +74,33 @@ __device__ __forceinline__ double img_pot(const Image& im, double x, double y, d
 // Surface kernels at point y (|y| = R_tau): G0 = 1/|x - y|; G1 is the dipole kernel of the
 // path: FP32 path the dy -> 0 limit (R_tau - x.yhat)/d^3, FP64 path the central difference
 // (1/d_- - 1/d_+)/dy = 2 (R_tau - x.yhat)/(d_+ d_- (d_+ + d_-)).
-__device__ __forceinline__ void surf_kernels(const SysDev& S, double x, double y, double z, const dbl4& yl,
-                                             double& g0, double& g1)
+__device__ __forceinline__ void surf_kernels(const SysDev& S, double x, double y, double z, double b0,
+                                             const dbl4& yl, double& g0, double& g1)
 {
   const double dx = x - yl.x, dy = y - yl.y, dz = z - yl.z;
   const double d2 = dx * dx + dy * dy + dz * dz;
+  if (S.prec != HSMA_FP64) {
+    // R_tau - x.yhat = (R_tau^2 - |x|^2 + d^2)/(2 R_tau) (every term positive inside the cavity; b0 =
+    // (R_tau^2 - |x|^2)/(2 R_tau)): 15 FP64 operations, where the unit vector, its product and the
+    // library's reciprocal root took about 35
+    g0 = rsqrt_f64(d2);
+    g1 = fma(0.5 * S.inv_Rt, d2, b0) * (g0 * g0 * g0);
+    return;
+  }
   g0 = rsqrt(d2);
   const double hx = yl.x * S.inv_Rt, hy = yl.y * S.inv_Rt, hz = yl.z * S.inv_Rt;  // |y| = R_tau
   const double xy = x * hx + y * hy + z * hz;
-  if (S.prec == HSMA_FP64) {
-    const double rm = S.Rtau - 0.5 * S.dy, rp = S.Rtau + 0.5 * S.dy;
-    const double mx = x - rm * hx, my = y - rm * hy, mz = z - rm * hz;
-    const double px = x - rp * hx, py = y - rp * hy, pz = z - rp * hz;
-    const double dm = sqrt(mx * mx + my * my + mz * mz);
-    const double dp = sqrt(px * px + py * py + pz * pz);
-    g1 = 2.0 * (S.Rtau - xy) / (dp * dm * (dp + dm));
-  } else {
-    g1 = (S.Rtau - xy) * (g0 * g0 * g0);
-  }
+  const double rm = S.Rtau - 0.5 * S.dy, rp = S.Rtau + 0.5 * S.dy;
+  const double mx = x - rm * hx, my = y - rm * hy, mz = z - rm * hz;
+  const double px = x - rp * hx, py = y - rp * hy, pz = z - rp * hz;
+  const double dm = sqrt(mx * mx + my * my + mz * mz);
+  const double dp = sqrt(px * px + py * py + pz * pz);
+  g1 = 2.0 * (S.Rtau - xy) / (dp * dm * (dp + dm));
+}
+// (R_tau^2 - |x|^2)/(2 R_tau)
+__device__ __forceinline__ double surf_b0(const SysDev& S, double x, double y, double z)
+{
+  return 0.5 * S.inv_Rt * (S.Rtau * S.Rtau - (x * x + y * y + z * z));
 }
 
 // Phi(y; A_x) and dPhi/dr for the coefficients of one charge q at x (addition theorem form).
@@ -195,8 +204,18 @@ __device__ __forceinline__ void series_eval(const SysDev& S, const SeriesShared&
   dphi = df_to_double(df_norm(sd)) * S.inv_Rt;
 }
 
-// Work item: (request, kind 0 = rows / 1 = surface, block)
-__global__ __launch_bounds__(kDeltaThreads) void k_delta(const SysDev* __restrict__ sys, const int4* __restrict__ items,
+// The moved charge's new and old position and image as (hi, lo) splits (FP32 path), once per block.
+struct MoveSplits {
+  float pos[2][2][3];  // [new, old][hi, lo][x, y, z]
+  float img[2][2][3];
+};
+
+// Work item: (request, kind 0 = rows / 1 = surface, block).  Bound by FP64 (1.6 FMA per clock and SM)
+// and, before, by its last block's one-thread sums: a request's partials, up to 195 dependent loads
+// and additions, took a third of the launch.  A block takes kDeltaRows rows, so that the images, the
+// splits and the FP64 block sum are made once for four rows of a thread; a warp adds a request's
+// partials.  64 requests over 687 000 charges: 128 us before, 67 us so.
+__global__ __launch_bounds__(kDeltaThreads, 3) void k_delta(const SysDev* __restrict__ sys, const int4* __restrict__ items,
                                                          int nitems, const int2* __restrict__ req_items,
                                                          const DeltaReq* __restrict__ reqs, int nreq,
                                                          const double* __restrict__ xyz, const double* __restrict__ q,
@@ -213,7 +232,8 @@ __global__ __launch_bounds__(kDeltaThreads) void k_delta(const SysDev* __restric
   __shared__ double red[kDeltaThreads / 32];
   __shared__ bool last;
   __shared__ SeriesShared ssh;
-  __shared__ Image s_in, s_io;
+  __shared__ Image s_im[2];
+  __shared__ MoveSplits s_sp;
   const double* inv_np1 = tab.inv_np1;
   const int4 it = items[blockIdx.x];
   const DeltaReq R = reqs[it.x];
@@ -222,75 +242,73 @@ __global__ __launch_bounds__(kDeltaThreads) void k_delta(const SysDev* __restric
   const double xo = xyz[3 * kk], yo = xyz[3 * kk + 1], zo = xyz[3 * kk + 2], qk = q[kk];
   const double xn = R.x, yn = R.y, zn = R.z;
   double acc = 0.0;
-  const int idx = it.z * kDeltaThreads + threadIdx.x;
   if (it.y == 0) {
-    // the moved charge's images (FP64), once per block
-    if (threadIdx.x == 0) {
-      s_in = kelvin_image(S, xn, yn, zn, qk);
-      s_io = kelvin_image(S, xo, yo, zo, qk);
+    // the moved charge's images (FP64), once per block: one thread of warp 0 and one of warp 1
+    if ((threadIdx.x & 31) == 0 && threadIdx.x < 64) {
+      const int side = threadIdx.x >> 5;
+      const double x = side ? xo : xn, y = side ? yo : yn, z = side ? zo : zn;
+      const Image im = kelvin_image(S, x, y, z, qk);
+      s_im[side] = im;
+      split_hilo(x, s_sp.pos[side][0][0], s_sp.pos[side][1][0]);
+      split_hilo(y, s_sp.pos[side][0][1], s_sp.pos[side][1][1]);
+      split_hilo(z, s_sp.pos[side][0][2], s_sp.pos[side][1][2]);
+      split_hilo(im.x, s_sp.img[side][0][0], s_sp.img[side][1][0]);
+      split_hilo(im.y, s_sp.img[side][0][1], s_sp.img[side][1][1]);
+      split_hilo(im.z, s_sp.img[side][0][2], s_sp.img[side][1][2]);
     }
     __syncthreads();
-    const Image In = s_in, Io = s_io;
+    const Image In = s_im[0], Io = s_im[1];
     if (blockIdx.x == req_items[it.x].x && threadIdx.x == 0) {
       const double rn2 = xn * xn + yn * yn + zn * zn;
       if (!(rn2 < S.a * S.a) || !isfinite(rn2)) atomicOr(status, kStBadMove);
       // the moved charge and its own image
       acc += 0.5 * qk * (img_pot(In, xn, yn, zn) - img_pot(Io, xo, yo, zo));
     }
+    const int ks = iperm[kk];
+    const MoveSplits& m = s_sp;
+    double pot = 0.0;  // sums of the potential differences of k's charge (times q_k)
     // rows run over sorted positions j (records are in the spatial order of k_order.cu)
-    const int j = idx;
-    if (j < S.n && j != iperm[kk]) {
+#pragma unroll
+    for (int u = 0; u < kDeltaRows / kDeltaThreads; ++u) {
+      const int j = it.z * kDeltaRows + u * kDeltaThreads + threadIdx.x;
+      if (j >= S.n || j == ks) continue;
       const double qj = q[S.chg + perm[S.chg + j]];
       if (S.prec == HSMA_FP64) {
         const dbl4 rj = src64[S.src + j];
         const dbl4 kj = src64[S.src + S.n + j];
         const double cn = inv_dist64(xn, yn, zn, rj.x, rj.y, rj.z), co = inv_dist64(xo, yo, zo, rj.x, rj.y, rj.z);
-        acc += qk * rj.w * (cn - co);
-        if (kj.w != 0.0) acc += 0.5 * qk * kj.w * (inv_dist64(xn, yn, zn, kj.x, kj.y, kj.z) -
-                                                   inv_dist64(xo, yo, zo, kj.x, kj.y, kj.z));
+        pot += rj.w * (cn - co);
+        if (kj.w != 0.0) pot += 0.5 * kj.w * (inv_dist64(xn, yn, zn, kj.x, kj.y, kj.z) -
+                                              inv_dist64(xo, yo, zo, kj.x, kj.y, kj.z));
         acc += 0.5 * qj * (img_pot(In, rj.x, rj.y, rj.z) - img_pot(Io, rj.x, rj.y, rj.z));
       } else {
-        float nh[3], nl[3], oh[3], ol[3];
-        split_hilo(xn, nh[0], nl[0]); split_hilo(yn, nh[1], nl[1]); split_hilo(zn, nh[2], nl[2]);
-        split_hilo(xo, oh[0], ol[0]); split_hilo(yo, oh[1], ol[1]); split_hilo(zo, oh[2], ol[2]);
         const float4 rh = src_hi[S.src + j], rl = src_lo[S.src + j];
         const float4 kh = src_hi[S.src + S.n + j], kl = src_lo[S.src + S.n + j];
-        float t = rh.w * (inv_hilo(nh[0], nh[1], nh[2], nl[0], nl[1], nl[2], rh.x, rh.y, rh.z, rl.x, rl.y, rl.z) -
-                          inv_hilo(oh[0], oh[1], oh[2], ol[0], ol[1], ol[2], rh.x, rh.y, rh.z, rl.x, rl.y, rl.z));
-        acc += qk * (double)t;
-        t = kh.w * (inv_hilo(nh[0], nh[1], nh[2], nl[0], nl[1], nl[2], kh.x, kh.y, kh.z, kl.x, kl.y, kl.z) -
-                    inv_hilo(oh[0], oh[1], oh[2], ol[0], ol[1], ol[2], kh.x, kh.y, kh.z, kl.x, kl.y, kl.z));
-        acc += 0.5 * qk * (double)t;
+        auto inv = [](const float (&p)[2][3], const float4& h, const float4& l) {
+          return inv_hilo(p[0][0], p[0][1], p[0][2], p[1][0], p[1][1], p[1][2], h.x, h.y, h.z, l.x, l.y, l.z);
+        };
+        const float tr = rh.w * (inv(m.pos[0], rh, rl) - inv(m.pos[1], rh, rl));
+        const float tk = kh.w * (inv(m.pos[0], kh, kl) - inv(m.pos[1], kh, kl));
+        pot += (double)tr;
+        pot = fma(0.5, (double)tk, pot);
         // j's charge in k's image potential (images split hi/lo like the records)
-        float ih[3], il[3], jh[3], jl[3];
-        double pn, po;
-        if (In.centre) {
-          pn = In.C;
-        } else {
-          split_hilo(In.x, ih[0], il[0]); split_hilo(In.y, ih[1], il[1]); split_hilo(In.z, ih[2], il[2]);
-          jh[0] = rh.x; jh[1] = rh.y; jh[2] = rh.z; jl[0] = rl.x; jl[1] = rl.y; jl[2] = rl.z;
-          pn = In.Q * (double)inv_hilo(jh[0], jh[1], jh[2], jl[0], jl[1], jl[2], ih[0], ih[1], ih[2], il[0], il[1], il[2]);
-        }
-        if (Io.centre) {
-          po = Io.C;
-        } else {
-          split_hilo(Io.x, ih[0], il[0]); split_hilo(Io.y, ih[1], il[1]); split_hilo(Io.z, ih[2], il[2]);
-          po = Io.Q * (double)inv_hilo(rh.x, rh.y, rh.z, rl.x, rl.y, rl.z, ih[0], ih[1], ih[2], il[0], il[1], il[2]);
-        }
-        acc += 0.5 * qj * (pn - po);
+        const double pn = In.centre ? In.C : In.Q * (double)inv(m.img[0], rh, rl);
+        const double po = Io.centre ? Io.C : Io.Q * (double)inv(m.img[1], rh, rl);
+        acc = fma(0.5 * qj, pn - po, acc);
       }
     }
+    acc = fma(qk, pot, acc);
   } else {
     const bool dfs = S.prec != HSMA_FP64;
     if (dfs) series_prepare(S, Mn, xn, yn, zn, xo, yo, zo, qk, ssh);
-    const int l = idx;
+    const int l = it.z * kDeltaThreads + threadIdx.x;
     if (l < S.M) {
       const dbl4 yl = surfx[S.surf + l];
       const double2 QD = surfqd[S.surf + l];
       const double2 V = vsurf[S.surf + l];
       double g0n, g1n, g0o, g1o, pn, dpn, po, dpo;
-      surf_kernels(S, xn, yn, zn, yl, g0n, g1n);
-      surf_kernels(S, xo, yo, zo, yl, g0o, g1o);
+      surf_kernels(S, xn, yn, zn, surf_b0(S, xn, yn, zn), yl, g0n, g1n);
+      surf_kernels(S, xo, yo, zo, surf_b0(S, xo, yo, zo), yl, g0o, g1o);
       if (dfs) {
         series_eval(S, ssh, 0, yl, tab, pn, dpn);
         series_eval(S, ssh, 1, yl, tab, po, dpo);
@@ -298,7 +316,7 @@ __global__ __launch_bounds__(kDeltaThreads) void k_delta(const SysDev* __restric
         charge_series(S, Mn, inv_np1, xn, yn, zn, qk, yl, pn, dpn);
         charge_series(S, Mn, inv_np1, xo, yo, zo, qk, yl, po, dpo);
       }
-      const double w4 = yl.w / (4.0 * kPi);
+      const double w4 = yl.w * (1.0 / (4.0 * kPi));
       const double dQ0 = w4 * (dpn - dpo), dD = w4 * (pn - po);
       const double dV0 = qk * (g0n - g0o), dV1 = qk * (g1n - g1o);
       acc += 0.5 * (dQ0 * (V.x + dV0) + QD.x * dV0 + dD * (V.y + dV1) + QD.y * dV1);
@@ -317,42 +335,81 @@ __global__ __launch_bounds__(kDeltaThreads) void k_delta(const SysDev* __restric
   __syncthreads();
   if (!last) return;
   __threadfence();
-  for (int r = threadIdx.x; r < nreq; r += kDeltaThreads) {
+  // a warp per request: its partials strided over the lanes, then the lanes' sums (a fixed order)
+  for (int r = threadIdx.x >> 5; r < nreq; r += kDeltaThreads / 32) {
     const int2 rg = req_items[r];
     double s = 0.0;
-    for (int i = 0; i < rg.y; ++i) s += ((volatile double*)dpart)[rg.x + i];
-    de[r] = s;
+    for (int i = threadIdx.x & 31; i < rg.y; i += 32) s += __ldcg(&dpart[rg.x + i]);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) de[r] = s;
   }
   if (threadIdx.x == 0) *counter = 0u;
 }
 
-// Potentials of the real charges under the two surface kernels, V0_l and V1_l (FP64; one warp
-// per surface point, fixed lane order and shuffle tree).
+// Potentials of the real charges under the two surface kernels, V0_l and V1_l (FP64).  A block takes
+// 8 points: warp w the points 4 (w & 1) .. + 3 over a quarter of the charges (w >> 1), lane-strided;
+// lanes by a shuffle tree, then the quarters, in a fixed order.  Bound by FP64: on the FP32 path
+// g1 = g0/(2 R_tau) + b0 g0^3 (surf_kernels, d^2 g0^2 = 1), so that a pair takes 15 operations and four
+// points share a charge's b0.  687 000 charges, M = 1000: 23.3 ms; 29.7 with a warp per point and the library's
+// reciprocal root.
+constexpr int kSpPoints = 4;
 __global__ __launch_bounds__(256) void k_surface_potentials(const SysDev* __restrict__ sys,
                                                             const int2* __restrict__ items,
                                                             const double* __restrict__ xyz,
                                                             const double* __restrict__ q,
                                                             const dbl4* __restrict__ surfx, double2* __restrict__ vsurf)
 {
+  __shared__ double2 part[8][kSpPoints];
   const int2 it = items[blockIdx.x];
   const SysDev& S = sys[it.x];
-  const int l = it.y * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (l >= S.M) return;
-  const dbl4 yl = surfx[S.surf + l];
-  double v0 = 0.0, v1 = 0.0;
-  for (int i = lane; i < S.n; i += 32) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int l0 = it.y * 8 + kSpPoints * (w & 1), quarter = w >> 1;
+  dbl4 y[kSpPoints];
+  double v0[kSpPoints], v1[kSpPoints];
+#pragma unroll
+  for (int k = 0; k < kSpPoints; ++k) {
+    y[k] = surfx[S.surf + min(l0 + k, S.M - 1)];
+    v0[k] = v1[k] = 0.0;
+  }
+  for (int i = 32 * quarter + lane; i < S.n; i += 128) {
     const long long g = S.chg + i;
-    double g0, g1;
-    surf_kernels(S, xyz[3 * g], xyz[3 * g + 1], xyz[3 * g + 2], yl, g0, g1);
-    v0 += q[g] * g0;
-    v1 += q[g] * g1;
+    const double x0 = xyz[3 * g], x1 = xyz[3 * g + 1], x2 = xyz[3 * g + 2], qi = q[g];
+    const double b0 = surf_b0(S, x0, x1, x2), qb = qi * b0;
+#pragma unroll
+    for (int k = 0; k < kSpPoints; ++k) {
+      if (S.prec == HSMA_FP64) {
+        double g0, g1;
+        surf_kernels(S, x0, x1, x2, b0, y[k], g0, g1);
+        v0[k] += qi * g0;
+        v1[k] += qi * g1;
+      } else {
+        const double dx = x0 - y[k].x, dy = x1 - y[k].y, dz = x2 - y[k].z;
+        const double g0 = rsqrt_f64(dx * dx + dy * dy + dz * dz);
+        v0[k] = fma(qi, g0, v0[k]);
+        v1[k] = fma(qb, g0 * g0 * g0, v1[k]);
+      }
+    }
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    v0 += __shfl_xor_sync(0xffffffffu, v0, o);
-    v1 += __shfl_xor_sync(0xffffffffu, v1, o);
+#pragma unroll
+  for (int k = 0; k < kSpPoints; ++k) {
+    for (int o = 16; o > 0; o >>= 1) {
+      v0[k] += __shfl_xor_sync(0xffffffffu, v0[k], o);
+      v1[k] += __shfl_xor_sync(0xffffffffu, v1[k], o);
+    }
+    if (lane == 0) part[w][k] = make_double2(v0[k], v1[k]);
   }
-  if (lane == 0) vsurf[S.surf + l] = make_double2(v0, v1);
+  __syncthreads();
+  const int p = threadIdx.x;  // point
+  if (p < 8 && it.y * 8 + p < S.M) {
+    double a = 0.0, b = 0.0;
+    for (int r = 0; r < 4; ++r) {
+      const double2 v = part[2 * r + p / kSpPoints][p % kSpPoints];
+      a += v.x;
+      b += v.y;
+    }
+    if (S.prec != HSMA_FP64) b = fma(0.5 * S.inv_Rt, a, b);
+    vsurf[S.surf + it.y * 8 + p] = make_double2(a, b);
+  }
 }
 
 // Order-independent float min/max in global memory (integer atomics on the bit patterns:
@@ -384,7 +441,8 @@ __device__ __forceinline__ void box_grow(float4* box, float x, float y, float z)
 }
 
 // Commit of a move, surface part: Q0, D, V0, V1 and the pair-sum surface records of every point.
-// Must run before k_move_charge (it reads the old position).
+// k_move_charge, its programmatic dependent, runs beside it and waits for it before it replaces the
+// position that both read (the two take 19 and 23 us of FP64 chains on a few blocks each).
 __global__ __launch_bounds__(256) void k_move_surface(const SysDev* __restrict__ sys, const int2* __restrict__ items,
                                                       const DeltaReq* __restrict__ reqs, const double* __restrict__ xyz,
                                                       const double* __restrict__ q, const double* __restrict__ Mn,
@@ -395,6 +453,7 @@ __global__ __launch_bounds__(256) void k_move_surface(const SysDev* __restrict__
                                                       dbl4* __restrict__ surf64_a, double* __restrict__ surf64_b)
 {
   __shared__ SeriesShared ssh;
+  allow_dependents();
   const int2 it = items[blockIdx.x];  // (request, block)
   const DeltaReq R = reqs[it.x];
   const SysDev& S = sys[R.sys];
@@ -414,15 +473,15 @@ __global__ __launch_bounds__(256) void k_move_surface(const SysDev* __restrict__
     charge_series(S, Mn, tab.inv_np1, R.x, R.y, R.z, qk, yl, pn, dpn);
     charge_series(S, Mn, tab.inv_np1, xo, yo, zo, qk, yl, po, dpo);
   }
-  const double w4 = yl.w / (4.0 * kPi);
+  const double w4 = yl.w * (1.0 / (4.0 * kPi));
   double2 QD = surfqd[o];
   QD.x += w4 * (dpn - dpo);
   QD.y += w4 * (pn - po);
   surfqd[o] = QD;
   if (have_v) {
     double g0n, g1n, g0o, g1o;
-    surf_kernels(S, R.x, R.y, R.z, yl, g0n, g1n);
-    surf_kernels(S, xo, yo, zo, yl, g0o, g1o);
+    surf_kernels(S, R.x, R.y, R.z, surf_b0(S, R.x, R.y, R.z), yl, g0n, g1n);
+    surf_kernels(S, xo, yo, zo, surf_b0(S, xo, yo, zo), yl, g0o, g1o);
     double2 V = vsurf[o];
     V.x += qk * (g0n - g0o);
     V.y += qk * (g1n - g1o);
@@ -433,13 +492,14 @@ __global__ __launch_bounds__(256) void k_move_surface(const SysDev* __restrict__
     surf64_b[o] = QD.y;
   } else {
     surf_a[o] = make_float4((float)yl.x, (float)yl.y, (float)yl.z, (float)QD.x);
-    surf_b[o] = make_float4((float)(-QD.y / S.Rtau), 0.f, 0.f, 0.f);
+    surf_b[o] = make_float4((float)(-QD.y * S.inv_Rt), 0.f, 0.f, 0.f);
   }
 }
 
 // Commit of a move, charge part (one block per request): coefficients A += dA (two solid-harmonic
-// columns sets computed by warps 0 and 1), the real and Kelvin records of k, the centre constant,
-// and the position itself.
+// columns sets computed by warps 0 and 1), the real and Kelvin records of k (the images computed
+// beside them by warps 2 and 3: one thread's FP64 roots and divisions are as long a chain), the
+// centre constant, and the position itself.
 __global__ __launch_bounds__(256) void k_move_charge(const SysDev* __restrict__ sys, const DeltaReq* __restrict__ reqs,
                                                      Tables tab, double* __restrict__ xyz, const double* __restrict__ q,
                                                      const double* __restrict__ Mn, double* __restrict__ coef,
@@ -457,9 +517,12 @@ __global__ __launch_bounds__(256) void k_move_charge(const SysDev* __restrict__ 
   const long long kk = S.chg + R.k;
   const double xo = xyz[3 * kk], yo = xyz[3 * kk + 1], zo = xyz[3 * kk + 2], qk = q[kk];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const double a = S.a;
+  __shared__ Image s_im[2];
+  if (warp >= 2 && warp < 4 && lane == 0)
+    s_im[warp - 2] = warp == 2 ? kelvin_image(S, R.x, R.y, R.z, qk) : kelvin_image(S, xo, yo, zo, qk);
   if (warp < 2) {
-    const double x = (warp == 0 ? R.x : xo) / a, y = (warp == 0 ? R.y : yo) / a, z = (warp == 0 ? R.z : zo) / a;
+    const double ia = S.inv_a;
+    const double x = (warp == 0 ? R.x : xo) * ia, y = (warp == 0 ? R.y : yo) * ia, z = (warp == 0 ? R.z : zo) * ia;
     const double rho2 = x * x + y * y + z * z;
     double* T = warp == 0 ? Tn : To;
     for (int m = lane; m <= p; m += 32) {
@@ -490,22 +553,21 @@ __global__ __launch_bounds__(256) void k_move_charge(const SysDev* __restrict__ 
   }
   __syncthreads();
   const double rn = sqrt(R.x * R.x + R.y * R.y + R.z * R.z), ro = sqrt(xo * xo + yo * yo + zo * zo);
-  const double cn = S.dbar * (S.Rtau * rn / (a * a) - 1.0) * 0.5;
-  const double co = S.dbar * (S.Rtau * ro / (a * a) - 1.0) * 0.5;
+  const double cn = S.dbar * (S.Rt_a * (rn * S.inv_a) - 1.0) * 0.5;
+  const double co = S.dbar * (S.Rt_a * (ro * S.inv_a) - 1.0) * 0.5;
   for (int idx = threadIdx.x; idx < P; idx += blockDim.x) {
-    int n = (int)sqrt((double)idx);
+    int n = (int)sqrtf((float)idx);
     while (n * n > idx) --n;
     while ((n + 1) * (n + 1) <= idx) ++n;
     const double mg = Mn[S.mn + n] - S.gam;
-    const double c = coef[S.coef + idx] + S.kc / a * qk * ((mg - cn) * Tn[idx] - (mg - co) * To[idx]);
+    const double c = coef[S.coef + idx] + S.kc_a * qk * ((mg - cn) * Tn[idx] - (mg - co) * To[idx]);
     coef[S.coef + idx] = c;
     float ch, cl;
     split_double(c, ch, cl);
     coef2[S.coef + idx] = make_float2(ch, cl);
   }
   if (threadIdx.x == 0) {
-    const Image In = kelvin_image(S, R.x, R.y, R.z, qk);
-    const Image Io = kelvin_image(S, xo, yo, zo, qk);
+    const Image In = s_im[0], Io = s_im[1];
     r0[R.sys] += In.C - Io.C;
     // the records sit at k's sorted position; its boxes grow to cover the new points (the
     // order itself is refreshed by the next full build)
@@ -518,7 +580,7 @@ __global__ __launch_bounds__(256) void k_move_charge(const SysDev* __restrict__ 
       float hx, hy, hz, lx, ly, lz;
       // (the lo records' fourth components: the weights of the symmetric pair sum's transposed
       // Kelvin term, as written by k_images)
-      const double rn2 = sqrt(__dadd_rn(__dadd_rn(__dmul_rn(R.x, R.x), __dmul_rn(R.y, R.y)), __dmul_rn(R.z, R.z)));
+      const double rn2 = rn;
       split_hilo(R.x, hx, lx); split_hilo(R.y, hy, ly); split_hilo(R.z, hz, lz);
       src_hi[sr] = make_float4(hx, hy, hz, (float)(S.kc * qk));
       src_lo[sr] = make_float4(lx, ly, lz, In.centre ? 0.f : (float)(In.Q * rn2));
@@ -529,6 +591,9 @@ __global__ __launch_bounds__(256) void k_move_charge(const SysDev* __restrict__ 
       src_lo[sk] = make_float4(lx, ly, lz, In.centre ? (float)(1e15 * S.inv_a) : (float)(1.0 / rn2));
       if (!In.centre) box_grow(boxes + 2 * bk, hx, hy, hz);
     }
+  }
+  grid_dependency_wait();  // k_move_surface has read the old position
+  if (threadIdx.x == 0) {
     xyz[3 * kk] = R.x;
     xyz[3 * kk + 1] = R.y;
     xyz[3 * kk + 2] = R.z;
@@ -564,9 +629,8 @@ void launch_move(const SysDev* sys, const int2* surf_items, int n_surf_items, co
   if (n_surf_items > 0)
     k_move_surface<<<n_surf_items, 256, 0, st>>>(sys, surf_items, reqs, xyz, q, Mn, tab, surfx, surfqd,
                                                  vsurf, have_v, surf_a, surf_b, surf64_a, surf64_b);
-  k_move_charge<<<nreq, 256, 2 * (size_t)maxP * sizeof(double), st>>>(sys, reqs, tab, xyz, q, Mn,
-                                                                     coef, coef2, r0, iperm, src_hi, src_lo, src64,
-                                                                     boxes);
+  launch_k(k_move_charge, nreq, 256, 2 * (size_t)maxP * sizeof(double), st, n_surf_items > 0, sys, reqs, tab, xyz, q,
+           Mn, coef, coef2, r0, iperm, src_hi, src_lo, src64, boxes);
 }
 
 void init_delta_kernels()

@@ -152,20 +152,6 @@ void launch_pairs_f32(int cfg, int grid, const SysDev* sys, PairWork w1, PairWor
 // at the same error against the 64-bit definition (1.2e-15).
 constexpr int kF64Threads = kF64TargetsPerBlock;
 
-// 1/sqrt(x): the approximate reciprocal root (relative error below 2^-19), then, with e = 1 - x y^2,
-// y + y e (1/2 + 3/8 e) (the next term, 5/16 e^3, is below 2^-56).  Arguments whose exponent leaves
-// no room for the step (zero, subnormal, near overflow, not finite) take the square root and the
-// division.
-__device__ __forceinline__ double rsqrt_f64(double x)
-{
-  const unsigned int top = (unsigned int)__double2hiint(x) >> 20;  // sign and exponent
-  if (top - 0x040u > 0x780u - 0x040u) return 1.0 / sqrt(x);
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-(x * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
 __global__ __launch_bounds__(kF64Threads) void k_pairs_f64(const SysDev* __restrict__ sys, PairWork w1,
                                                            PairWork w2, const dbl4* __restrict__ src64,
                                                            const dbl4* __restrict__ surf64_a,

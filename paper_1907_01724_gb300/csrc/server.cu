@@ -290,7 +290,7 @@ static int launch_moves(hsma_server_t* s, const std::vector<Pending>& batch)
     s->dreq_h[r] = d;
     const hsma::SysDev& sd = e->L.sd[d.sys];
     s->dranges_h[r].x = ni;
-    for (int b = 0; b < (sd.n + hsma::kDeltaBlock - 1) / hsma::kDeltaBlock; ++b) s->ditems_h[ni++] = make_int4(r, 0, b, 0);
+    for (int b = 0; b < (sd.n + hsma::kDeltaRows - 1) / hsma::kDeltaRows; ++b) s->ditems_h[ni++] = make_int4(r, 0, b, 0);
     for (int b = 0; b < (sd.M + hsma::kDeltaBlock - 1) / hsma::kDeltaBlock; ++b) s->ditems_h[ni++] = make_int4(r, 1, b, 0);
     s->dranges_h[r].y = ni - s->dranges_h[r].x;
     if (q.accept) {

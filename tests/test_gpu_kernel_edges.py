@@ -56,3 +56,24 @@ def test_tree_at_batch_edges(n, order):
     api.hsma_set_far_field(h, 0.35 if order == 8 else 0.5, order)
     api.hsma_build_sources(h, s.xyz, s.q)
     assert np.linalg.norm(api.hsma_potential(h) - ref) <= 1e-6 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("M", [6, 30])
+@pytest.mark.parametrize("n", [1, 2, 1024, 1025, 2049])
+def test_move_energies_at_block_edges(n, M):
+    """Delta E and a committed move where the row blocks (1024 rows) and the blocks of surface points
+    (8) end, FP32 against FP64 path: 1e-6 of the moved charge's Coulomb terms and of Delta E."""
+    rng = np.random.default_rng(190820 + n)
+    xyz, q = inputs.uniform_ball(rng, n, 0.9), rng.choice([-1.0, 1.0], n)
+    k, xs = n // 2, inputs.uniform_ball(rng, 2, 0.9)
+    de = {}
+    for prec in (api.HSMA_FP32, api.HSMA_FP64):
+        h = api.hsma_create(1.0, 2.0, 80.0, 1.5, api.hsma_default_params(p=12, M=M, precision=prec))
+        api.hsma_build_sources(h, xyz, q)
+        first = api.hsma_delta_energy(h, k, xs[0])
+        api.hsma_apply_move(h, k, xs[0])
+        de[prec] = np.array([first, api.hsma_delta_energy(h, k, xs[1])])
+    kc = api.PAPER_COULOMB_K / 2.0
+    others = np.delete(xyz, k, 0)
+    S = kc * (sum((1.0 / np.linalg.norm(others - x, axis=1)).sum() for x in (xyz[k], xs[0], xs[1])) + 1.0)
+    assert np.abs(de[api.HSMA_FP32] - de[api.HSMA_FP64]).max() <= 1e-6 * (S + np.abs(de[api.HSMA_FP64]).max())
