@@ -591,7 +591,8 @@ __global__ __launch_bounds__(32 * kFarWarps) void k_tree_far(TreeView t)
 // the columns 2k, 2k + 1 (FFMA2 / FMUL2): per two coefficients one 16-byte shared load, the two
 // factors of Q_{n-2}, three operations of the recurrence and two of the sums -- 3.5 instructions a
 // coefficient where the recurrence on (Re, Im) took 5.  The columns run in two groups so that the state
-// (two rows and the sums) fits the registers of 24 warps per SM.  The evaluation is issue-bound
+// (two rows and the sums) fits the registers of 24 warps per SM (one group spills: N = 1e6 22.4 ms at 16
+// warps; three groups at 28 warps 20.1).  The evaluation is issue-bound
 // (76 % of the slots): with this series, the direct sums relative to the node's centre and one
 // reduction for the three tests of a node it takes 1.75 ms at N = 1e5 and 19.9 ms at N = 1e6 (theta =
 // 0.5, order 12; 2.47 and 24.2 ms before), at the same error (7.6e-8 at N = 1e5).
@@ -646,38 +647,37 @@ __device__ __forceinline__ void horner(float& sr, float& si, float zx, float zy,
   sr = nr;
 }
 
+// Column pairs K0..K1 - 1 of the series, added to the Horner sum (s <- s z^(2 (K1 - K0)) + ...); the
+// real column m = 0 (K0 = 0) is returned and left out.
+template <int P, int K0, int K1>
+__device__ __forceinline__ float series_add(const float4* M, float wz, float i2, float ri, int q, float px, float py,
+                                            float& sr, float& si)
+{
+  if (K0 > 0 && q < 2 * K0) return 0.f;
+  float2 CR[K1 - K0], CI[K1 - K0];
+  series_group<P, K0, K1>(M, wz, i2, ri, q, CR, CI);
+#pragma unroll
+  for (int k = K1 - K0 - 1; k >= 0; --k) {
+    horner(sr, si, px, py, CR[k].y, CI[k].y);
+    if (K0 + k > 0) horner(sr, si, px, py, CR[k].x, CI[k].x);
+  }
+  return CR[0].x;
+}
+
 template <int P>
 __device__ __forceinline__ float m2p(const float4* M, float4 gc, float4 th, float4 tl, int q)
 {
-  constexpr int KP = P / 2 + 1;              // column pairs
-  constexpr int KS = P <= 8 ? KP : P / 4;    // first pair of the second group
+  constexpr int KP = P / 2 + 1;  // column pairs
   const float ir = inv_unit(gc.w);
   const float ux = ((th.x - gc.x) + tl.x) * ir, uy = ((th.y - gc.y) + tl.y) * ir, uz = ((th.z - gc.z) + tl.z) * ir;
   const float r2 = ux * ux + uy * uy + uz * uz;
   const float i2 = __fdividef(1.f, r2), ri = rsqrt_mufu(r2);
   const float px = ux * i2, py = uy * i2, wz = uz * i2;
   float sr = 0.f, si = 0.f;
-  if constexpr (KS < KP) {
-    if (q >= 2 * KS) {
-      float2 CR[KP - KS], CI[KP - KS];
-      series_group<P, KS, KP>(M, wz, i2, ri, q, CR, CI);
-#pragma unroll
-      for (int k = KP - KS - 1; k >= 0; --k) {
-        horner(sr, si, px, py, CR[k].y, CI[k].y);
-        horner(sr, si, px, py, CR[k].x, CI[k].x);
-      }
-    }
-  }
-  float2 CR[KS], CI[KS];
-  series_group<P, 0, KS>(M, wz, i2, ri, q, CR, CI);
-#pragma unroll
-  for (int k = KS - 1; k >= 1; --k) {
-    horner(sr, si, px, py, CR[k].y, CI[k].y);
-    horner(sr, si, px, py, CR[k].x, CI[k].x);
-  }
-  horner(sr, si, px, py, CR[0].y, CI[0].y);
-  // Re(S z) twice, and the real column m = 0
-  return fmaf(2.f, fmaf(sr, px, -si * py), CR[0].x) * ir;
+  // groups of column pairs, the highest first
+  series_add<P, P / 4, KP>(M, wz, i2, ri, q, px, py, sr, si);
+  const float c0 = series_add<P, 0, P / 4>(M, wz, i2, ri, q, px, py, sr, si);
+  return fmaf(2.f, fmaf(sr, px, -si * py), c0) * ir;
 }
 
 // phi at the target of the far images' expansion (|x| < a)
