@@ -77,3 +77,18 @@ def test_move_energies_at_block_edges(n, M):
     others = np.delete(xyz, k, 0)
     S = kc * (sum((1.0 / np.linalg.norm(others - x, axis=1)).sum() for x in (xyz[k], xs[0], xs[1])) + 1.0)
     assert np.abs(de[api.HSMA_FP32] - de[api.HSMA_FP64]).max() <= 1e-6 * (S + np.abs(de[api.HSMA_FP64]).max())
+
+
+@pytest.mark.parametrize("n, M", [(9000, 70), (13001, 2000), (16385, 130)])
+def test_field_chunks_merged(n, M):
+    """The FP32 field pass at sizes where several source chunks make one field chunk, the last of them
+    not full, against the FP64 field pass: 1e-6 norm-wise for each of its outputs."""
+    rng = np.random.default_rng(190830 + n)
+    xyz, q = inputs.uniform_ball(rng, n, 1.0), rng.choice([-1.0, 1.0], n)
+    out = {}
+    for prec in (api.HSMA_FP32, api.HSMA_FP64):
+        h = api.hsma_create(1.0, 2.0, 80.0, 1.5, api.hsma_default_params(p=12, M=M, precision=prec))
+        api.hsma_build_sources(h, xyz, q)
+        out[prec] = [api.hsma_field(h, w) for w in (api.HSMA_TOTAL, api.HSMA_COULOMB, api.HSMA_REACTION)]
+    for a, b in zip(out[api.HSMA_FP32], out[api.HSMA_FP64]):
+        assert np.linalg.norm(a - b) <= 1e-6 * np.linalg.norm(b)
