@@ -271,6 +271,14 @@ int Engine::make_field_items()
   return HSMA_OK;
 }
 
+// Share of the pair items that each system gets at least where systems are evaluated one at a time
+// (Engine::one_by_one): a launch over one system of a batch's few large items leaves most of the
+// workers idle for as long as its longest item takes (a block pair of 512 charges: 175 us).  The
+// request server, 64 chains of 500 to 50000 charges, 1000 requests, four seeds, in ms:
+//   share 0: 14.1 11.9 8.1 10.6;  1/8: 13.2 11.2 7.3 9.9;  1/4: 13.1 11.1 7.3 9.8;
+//   1/2: 13.4 11.5 7.2 10.0;  1: 13.8 11.5 7.6 10.2 (more partials and staging per pair)
+constexpr double kAloneShare = 0.25;
+
 // sizes_only: the workspace plan alone (the pair items are counted, not listed).
 Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_only) const
 {
@@ -365,7 +373,9 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_o
     d.n_tb = (int)((n + TB - 1) / TB);
     if (n > 0) {
       const double Ws = (double)n * (2.0 * n + 1.3 * sp.M);
-      const double items_s = std::max(1.0, std::round(desired * Ws / std::max(W, 1.0)));
+      double share = Ws / std::max(W, 1.0);
+      if (one_by_one && prec != HSMA_FP64) share = std::max(share, kAloneShare);
+      const double items_s = std::max(1.0, std::round(desired * share));
       if (prec == HSMA_FP64) {
         const int64_t chunks_total = std::max<int64_t>(1, (int64_t)std::ceil(items_s / d.n_tb));
         const int64_t per = (2 * n + sp.M + chunks_total - 1) / chunks_total;

@@ -129,6 +129,8 @@ class Engine {
   // far field of the real/Kelvin pair sums by the treecode of k_tree.cu (single FP32 system):
   // far_theta = 0 keeps the direct sum; takes effect at the next layout
   double far_theta = 0.0;
+  // the systems' pair sums are launched one system at a time (the server's full energies)
+  bool one_by_one = false;
   int far_order = 12;
   TreeView tree_view() const;
   cudaEvent_t ev_tree0 = nullptr, ev_tree1 = nullptr;  // around the tree evaluation

@@ -666,6 +666,7 @@ int hsma_server_create(int nchains, const double* a, const double* eps1, const d
   s->energy_slots = energy_slots;
   s->sm_frac = energy_sm_frac;
   s->e = new Engine();
+  s->e->one_by_one = true;
   s->e->spec = {s->specs[0]};
   int rc = s->e->init(params->device, nullptr, params->precision);
   if (rc) {

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import oracle
-from paper_1907_01724_gb300 import api, inputs
+from paper_1907_01724_gb300 import api, inputs, server
 
 pytestmark = pytest.mark.gpu
 
@@ -92,3 +92,27 @@ def test_field_chunks_merged(n, M):
         out[prec] = [api.hsma_field(h, w) for w in (api.HSMA_TOTAL, api.HSMA_COULOMB, api.HSMA_REACTION)]
     for a, b in zip(out[api.HSMA_FP32], out[api.HSMA_FP64]):
         assert np.linalg.norm(a - b) <= 1e-6 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("sizes", [(1, 127, 129, 9000), (511, 513, 2047, 16385), (64, 1000, 1024, 30000)])
+def test_server_energies_of_unequal_chains(sizes):
+    """Full energies of resident chains next to a much larger one (each chain's own share of pair
+    items, blocks of one group and ragged ones), against the FP64 path: |dE| <= f |q| |dphi| with
+    E = f q.phi and the FP32 path's bound |dphi| <= 1e-6 |phi|."""
+    rng = np.random.default_rng(190840 + sum(sizes))
+    chains = [inputs.System(1.0, 2.0, 80.0, 1.5, 12, 200, inputs.uniform_ball(rng, n, 1.0), rng.choice([-1.0, 1.0], n))
+              for n in sizes]
+    srv = server.Server(chains)
+    srv.hsma_server_load()
+    reqs = np.zeros(len(sizes), dtype=server.REQUEST)
+    reqs["id"] = reqs["chain"] = np.arange(len(sizes))
+    reqs["kind"] = server.REQ_ENERGY
+    res = srv.hsma_server_run(reqs)
+    assert (res["status"] == 0).all()
+    for r in res:
+        s = chains[r["chain"]]
+        h = api.hsma_create(s.a, s.eps1, s.eps2, s.kappa, api.hsma_default_params(p=s.p, M=s.M, precision=api.HSMA_FP64))
+        api.hsma_build_sources(h, s.xyz, s.q)
+        phi, E = api.hsma_potential(h), api.hsma_energy(h)[0]
+        f = abs(E / (s.q @ phi))
+        assert abs(r["value"] - E) <= 1e-6 * f * np.linalg.norm(s.q) * np.linalg.norm(phi)
