@@ -279,6 +279,9 @@ int Engine::make_field_items()
 //   1/2: 13.4 11.5 7.2 10.0;  1: 13.8 11.5 7.6 10.2 (more partials and staging per pair)
 constexpr double kAloneShare = 0.25;
 
+// Bytes of field partials above which a layout's field chunks are merged (half of the L2).
+constexpr double kFieldMergeBytes = 64e6;
+
 // sizes_only: the workspace plan alone (the pair items are counted, not listed).
 Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_only) const
 {
@@ -503,11 +506,12 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_o
         for (int b = 0; b < (spec[s].M + pts - 1) / pts; ++b) L.it3m.push_back(make_int2(s, b));
     }
   }
-  // field chunks: whole chunks of the pair pass, merged while four items per CTA slot are left; the
-  // list itself is made by the first field pass (make_field_items)
+  // field chunks: two chunks of the pair pass each where that leaves four to eight items per CTA slot
+  // (see k_field.cu); the list itself is made by the first field pass (make_field_items)
   L.TBf = TBf;
   const size_t fslots = (size_t)num_sms * std::max(prec == HSMA_FP64 ? occ_field64 : occ_field[cfg], 1);
-  const int merge = prec == HSMA_FP64 ? 1 : (int)std::max<size_t>(1, nfield / (4 * fslots));
+  const bool merges = prec != HSMA_FP64 && 32.0 * (double)part > kFieldMergeBytes;
+  const int merge = merges && nfield >= 8 * fslots && nfield < 16 * fslots ? 2 : 1;
   for (auto& d : L.sd) {
     d.fchunk = (int)std::min<int64_t>((int64_t)d.chunk * merge, std::max(d.chunk, d.n));
     d.fchunk_s = (int)std::min<int64_t>((int64_t)d.chunk_s * merge, std::max(d.chunk_s, d.M));

@@ -3,10 +3,12 @@
 // and dipole layers of the auxiliary sphere; Sec. 2.4, eqs. phicorrfinall and phirffinall),
 // differentiated term by term with the sources fixed, so that F_i = q_i E(x_i).
 //
-// Spatial order and the near/far box test are those of the potential pass.  A source chunk is a whole
-// number of its chunks (SysDev::fchunk), as many as leave four items per CTA slot: every chunk costs a
-// target 32 bytes of partials to write and to reduce (FP32, N = 20000, M = 2000: 527 us with the pair
-// pass's own chunks, 509 us merged; at two or eight items per slot 508 and 527).  Per (chunk, target)
+// Spatial order and the near/far box test are those of the potential pass.  A source chunk is one
+// chunk of the potential pass, or two where the partials would not stay in L2 and four to eight items
+// per CTA slot are left (SysDev::fchunk): every chunk costs a target 32 bytes of partials to write and
+// to reduce, and longer items end less evenly.  Fields and potentials, M = 2000, with one chunk and
+// with two: N = 13001 325 and 313 us, N = 20000 527 and 509 (608 and 602 for other charges),
+// N = 25000 860 and 882, N = 40000 1945 and 1985: merged up to about 20000.  Per (chunk, target)
 // the FP32 kernel writes two float4, the (hi, lo) two-sum pairs of (phi, Ex, Ey, Ez); the FP64 kernel
 // one (phi, Ex, Ey, Ez) in double.  k_reduce_field sums them in a fixed order (double-float on the
 // FP32 path) and maps them back to input order.
