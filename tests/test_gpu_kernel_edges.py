@@ -81,8 +81,8 @@ def test_move_energies_at_block_edges(n, M):
 
 @pytest.mark.parametrize("n, M", [(9000, 70), (13001, 2000), (16385, 130)])
 def test_field_chunks_merged(n, M):
-    """The FP32 field pass at sizes where several source chunks make one field chunk, the last of them
-    not full, against the FP64 field pass: 1e-6 norm-wise for each of its outputs."""
+    """The FP32 field pass where two source chunks make one field chunk, the last of them not full
+    (N = 13001), and next to that range, against the FP64 field pass: 1e-6 norm-wise for each output."""
     rng = np.random.default_rng(190830 + n)
     xyz, q = inputs.uniform_ball(rng, n, 1.0), rng.choice([-1.0, 1.0], n)
     out = {}
