@@ -29,6 +29,13 @@ __device__ __forceinline__ double rsqrt_f64(double x)
   return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
+// 1/s for the power of two s above x > 0: s = 2^(e + 1) for x in [2^e, 2^(e + 1)) (a unit of length
+// whose scalings are exact)
+__device__ __forceinline__ float inv_unit(float x)
+{
+  return __int_as_float(0x7e800000 - (__float_as_int(x) & 0x7f800000));
+}
+
 // 16-byte asynchronous global -> shared copy (both addresses 16-byte aligned), its commit group
 // and the wait for all but the N most recent groups.
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem)

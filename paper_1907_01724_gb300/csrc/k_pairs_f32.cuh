@@ -48,6 +48,9 @@
 // two multiply-adds a pair instead of the three-term product (10 FP32 operations and the rsqrt
 // instead of 13).  c_t is formed once per target and item, c_y (the rounding of a point's
 // coordinates) once per staged point, both in double-float; |c_t| >= tau a^2, so nothing cancels.
+// Lengths are in units of the power of two above a (exact scalings, once per target and staged
+// point): D' c_t in the caller's units, charge times length squared, leaves the FP32 range for a
+// cavity of nanometres in metres with charges in coulombs, where D' u, a charge, does not.
 //
 // Each target keeps an FP32 partial per group of boxes, folded into an (hi, lo) two-sum pair.
 
@@ -419,15 +422,16 @@ __global__ __launch_bounds__(NT, pair_min_blocks<NT, K>()) void k_pairs_f32(cons
     if (ch.type == 2) {
       // ---- surface item: one group of targets against a chunk of surface points ----------
       const int g0 = it.y * G;
-      const df Rt = df_make(S.f_a.x, S.f_a.y) * df_make(S.f_Rt_a.x, S.f_Rt_a.y);
+      const float iu = inv_unit(S.f_a.x);
+      const df Rt = df_make(S.f_a.x * iu, S.f_a.y * iu) * df_make(S.f_Rt_a.x, S.f_Rt_a.y);
       const df R2 = Rt * Rt;
       float tx[K], ty[K], tz[K], ct[K], H[K], L[K], acc[K];
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         const int i = g0 + k * 32 + lane;
         const float4 h = src_hi[S.src + (i < n ? i : g0)];
-        tx[k] = h.x; ty[k] = h.y; tz[k] = h.z;
-        ct[k] = 0.5f * (two_prod(h.x, h.x) + two_prod(h.y, h.y) + two_prod(h.z, h.z) - R2).hi;
+        tx[k] = h.x * iu; ty[k] = h.y * iu; tz[k] = h.z * iu;
+        ct[k] = 0.5f * (two_prod(tx[k], tx[k]) + two_prod(ty[k], ty[k]) + two_prod(tz[k], tz[k]) - R2).hi;
         H[k] = L[k] = acc[k] = 0.f;
       }
       const float4* ga = surf_a + ch.off;
@@ -449,8 +453,9 @@ __global__ __launch_bounds__(NT, pair_min_blocks<NT, K>()) void k_pairs_f32(cons
         }
         __syncwarp();  // the previous box's sums have read the buffer
         if (lane < cnt) {
-          const float cy = 0.5f * (two_prod(ra.x, ra.x) + two_prod(ra.y, ra.y) + two_prod(ra.z, ra.z) - R2).hi;
-          bA[lane] = make_float4(ra.x, ra.y, ra.z, fmaf(-0.5f, rd, ra.w));
+          const float yx = ra.x * iu, yy = ra.y * iu, yz = ra.z * iu;
+          const float cy = 0.5f * (two_prod(yx, yx) + two_prod(yy, yy) + two_prod(yz, yz) - R2).hi;
+          bA[lane] = make_float4(yx, yy, yz, fmaf(-0.5f, rd, ra.w));
           bQ[lane] = rd;
           bQ[lane + kBox] = -rd * cy;
         }
@@ -511,7 +516,7 @@ __global__ __launch_bounds__(NT, pair_min_blocks<NT, K>()) void k_pairs_f32(cons
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         const int i = g0 + k * 32 + lane;
-        if (i < n) out[i] = make_float2(H[k], L[k]);
+        if (i < n) out[i] = make_float2(H[k] * iu, L[k] * iu);
       }
       continue;
     }

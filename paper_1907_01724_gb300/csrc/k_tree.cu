@@ -77,12 +77,6 @@ __device__ __forceinline__ float2 get_moment(const float4* M, int P, int n, int 
   return make_float2(e[0], e[2]);
 }
 
-// 1/s of a node of radius rho > 0: s = 2^(e + 1) for rho in [2^e, 2^(e + 1))
-__device__ __forceinline__ float inv_unit(float rho)
-{
-  return __int_as_float(0x7e800000 - (__float_as_int(rho) & 0x7f800000));
-}
-
 // Whether a Kelvin record lies beyond kFarImageRel a (its high part, rounded without contraction,
 // so that every kernel classifies a record the same way).
 __device__ __forceinline__ bool far_image(float4 h, float rfar2)

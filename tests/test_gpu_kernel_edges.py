@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import oracle
-from paper_1907_01724_gb300 import api, inputs, server
+from paper_1907_01724_gb300 import api, batch, inputs, server
 
 pytestmark = pytest.mark.gpu
 
@@ -116,3 +116,22 @@ def test_server_energies_of_unequal_chains(sizes):
         phi, E = api.hsma_potential(h), api.hsma_energy(h)[0]
         f = abs(E / (s.q @ phi))
         assert abs(r["value"] - E) <= 1e-6 * f * np.linalg.norm(s.q) * np.linalg.norm(phi)
+
+
+@pytest.mark.parametrize("threads, k", [(128, 1), (64, 2), (64, 4), (128, 8)])
+@pytest.mark.parametrize("length, charge", [(2.0 ** -32, 2.0 ** -64), (2.0 ** 24, 2.0 ** 20)])
+def test_fp32_potentials_scale_with_lengths_and_charges(threads, k, length, charge):
+    """Lengths and charges scaled by powers of two (a cavity of nanometres in metres, with charges of
+    an electron in coulombs): every FP32 operation scales exactly while its result stays a normal
+    number, so the potentials are those of the unscaled cavity times charge / length; the FP32
+    path's own bound, 1e-6 norm-wise, is allowed."""
+    rng = np.random.default_rng(190850)
+    xyz, q = inputs.uniform_ball(rng, 300, 1.0), rng.choice([-1.0, 1.0], 300)
+    cfg = [tuple(c) for c in batch.pair_configs()].index((threads, k, 4))
+    phi = []
+    for s, t in ((1.0, 1.0), (length, charge)):
+        b = batch.from_systems([inputs.System(s, 2.0, 80.0, 1.5 / s, 12, 1000, s * xyz, t * q)])
+        b.hsma_batch_set_pair_config(cfg)
+        b.hsma_batch_build_sources(np.array([300]), s * xyz, t * q)
+        phi.append(b.hsma_batch_potential(api.HSMA_REACTION) * s / t)
+    assert np.linalg.norm(phi[1] - phi[0]) <= 1e-6 * np.linalg.norm(phi[0])
