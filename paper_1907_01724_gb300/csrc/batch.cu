@@ -326,13 +326,7 @@ static int batch_pot(hsma_batch_t* b, double* phi, int what, bool dev)
   bool wrote = false;
   int rc = b->e->potentials(od, &wrote);
   if (rc) return bfrom(b, rc);
-  if (dev) {
-    if (tot > 0 && !wrote) {
-      cudaError_t e = cudaMemcpyAsync(phi, src, 8 * tot, cudaMemcpyDeviceToDevice, b->e->stream);
-      if (e != cudaSuccess) return bfrom(b, b->e->cuda_fail(e, "copy phi"));
-    }
-    return HSMA_OK;
-  }
+  if (dev) return wrote ? HSMA_OK : bfrom(b, b->e->copy_to_device(src, tot, phi, "copy phi"));
   return bfrom(b, b->e->copy_to_host(src, tot, phi, wrote, phi_dev != nullptr));
 }
 
@@ -351,11 +345,7 @@ static int batch_field(hsma_batch_t* b, double* E, int what, bool dev)
   if (rc) return bfrom(b, rc);
   const double* src = what == HSMA_TOTAL ? b->e->Et_d : (what == HSMA_REACTION ? b->e->Er_d : b->e->Ec_d);
   if (!dev) return bfrom(b, b->e->copy_to_host(src, 3 * tot, E));
-  if (tot > 0) {
-    cudaError_t e = cudaMemcpyAsync(E, src, 24 * tot, cudaMemcpyDeviceToDevice, b->e->stream);
-    if (e != cudaSuccess) return bfrom(b, b->e->cuda_fail(e, "copy E"));
-  }
-  return HSMA_OK;
+  return bfrom(b, b->e->copy_to_device(src, 3 * tot, E, "copy E"));
 }
 
 int hsma_batch_set_overlap(hsma_batch_t* b, int on)

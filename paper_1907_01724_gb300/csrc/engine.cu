@@ -1486,6 +1486,19 @@ int Engine::check_status()
   return decode_status(*st_h);
 }
 
+// Copy count doubles of the current pass to a caller's device array, in the order of the caller's
+// stream: with a NULL stream after its legacy-stream work so far (which may still use the array)
+// and before what it enqueues next (the pass's own enter/leave pair ends before this copy).
+int Engine::copy_to_device(const double* src, int64_t count, double* dst, const char* what)
+{
+  if (count <= 0) return HSMA_OK;
+  enter();
+  const cudaError_t e = cudaMemcpyAsync(dst, src, 8 * (size_t)count, cudaMemcpyDeviceToDevice, stream);
+  if (e != cudaSuccess) return cuda_fail(e, what);
+  leave();
+  return HSMA_OK;
+}
+
 // Copy count doubles from the device to caller host memory through a pinned staging buffer,
 // with the energies (pinned mirror) and the status word in the same round trip, then decode the
 // status: one stream synchronisation instead of one per pageable copy.
@@ -1835,11 +1848,7 @@ int hsma_potential_device(hsma_t* h, double* phi_dev, int what)
   const hsma::OutDesc od{h->n > 0 ? phi_dev : nullptr, nullptr, nullptr, Engine::out_lane(what), 0};
   int rc = h->e->potentials(od, &wrote);
   if (rc) return from_engine(h, rc);
-  if (h->n > 0 && !wrote) {
-    cudaError_t e = cudaMemcpyAsync(phi_dev, src, 8 * h->n, cudaMemcpyDeviceToDevice, h->e->stream);
-    if (e != cudaSuccess) return from_engine(h, h->e->cuda_fail(e, "copy phi"));
-  }
-  return HSMA_OK;
+  return wrote ? HSMA_OK : from_engine(h, h->e->copy_to_device(src, h->n, phi_dev, "copy phi"));
 }
 
 static const double* pick_field(Engine* e, int what)
@@ -1862,11 +1871,7 @@ static int field_out(hsma_t* h, double* E, int what, bool dev)
   rc = h->e->field();
   if (rc) return from_engine(h, rc);
   if (!dev) return from_engine(h, h->e->copy_to_host(pick_field(h->e, what), 3 * h->n, E));
-  if (h->n > 0) {
-    cudaError_t e = cudaMemcpyAsync(E, pick_field(h->e, what), 24 * h->n, cudaMemcpyDeviceToDevice, h->e->stream);
-    if (e != cudaSuccess) return from_engine(h, h->e->cuda_fail(e, "copy E"));
-  }
-  return HSMA_OK;
+  return from_engine(h, h->e->copy_to_device(pick_field(h->e, what), 3 * h->n, E, "copy E"));
 }
 
 int hsma_field(hsma_t* h, double* E, int what) { return field_out(h, E, what, false); }

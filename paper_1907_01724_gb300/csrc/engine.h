@@ -92,6 +92,7 @@ class Engine {
   // (OutDesc), *wrote: whether a pass ran (and so wrote them)
   int potentials(const OutDesc& od = OutDesc{nullptr, nullptr, nullptr, 0, 0}, bool* wrote = nullptr);
   int set_outputs(const OutDesc& od);
+  int copy_to_device(const double* src, int64_t count, double* dst, const char* what);
   OutDesc* outdesc_d = nullptr;
   // Inputs of the next build pass (InDesc in the workspace): the caller's device arrays while a
   // build from them is pending (the pass reads them in place and copies them to xyz_d, q_d),

@@ -231,3 +231,36 @@ def test_page_locked_host_buffers(prec):
         assert rel(one, phi2[:sy[0].n]) <= tol
     finally:
         api.hsma_destroy(h)
+
+
+@pytest.mark.parametrize("kind", ["handle", "batch"])
+def test_device_outputs_follow_the_legacy_stream(kind):
+    """A handle without a stream of its own: device outputs that are copies (fields, and potentials of
+    a pass already run) are ordered before the caller's next legacy-stream work, which reads them here
+    while the pass is still running, and after its earlier work on the array."""
+    rng = np.random.default_rng(53)
+    s = inputs.System(1.0, 1.0, 78.5, 1.0, 12, 400, inputs.uniform_ball(rng, 20000, 1.0), rng.choice([-1.0, 1.0], 20000))
+    if kind == "handle":
+        h = api.hsma_create(s.a, s.eps1, s.eps2, s.kappa, api.hsma_default_params(p=s.p, M=s.M))
+        build, field, pot = (lambda: api.hsma_build_sources(h, s.xyz, s.q)), (lambda o: api.hsma_field(h, api.HSMA_TOTAL, out=o)), \
+            (lambda o: api.hsma_potential(h, api.HSMA_REACTION, out=o))
+        want = build() or (api.hsma_field(h, api.HSMA_TOTAL), api.hsma_potential(h, api.HSMA_REACTION))
+    else:
+        b = batch.from_systems([s])
+        n = np.array([s.n])
+        build, field, pot = (lambda: b.hsma_batch_build_sources(n, s.xyz, s.q)), (lambda o: b.hsma_batch_field(api.HSMA_TOTAL, out=o)), \
+            (lambda o: b.hsma_batch_potential(api.HSMA_REACTION, out=o))
+        want = build() or (b.hsma_batch_field(api.HSMA_TOTAL), b.hsma_batch_potential(api.HSMA_REACTION))
+    E = torch.empty((s.n, 3), dtype=torch.float64, device="cuda")
+    phi = torch.empty(s.n, dtype=torch.float64, device="cuda")
+    assert torch.cuda.current_stream().cuda_stream == 0
+    for _ in range(3):
+        build()
+        E.fill_(-7.0)
+        phi.fill_(-7.0)
+        field(E)
+        got_E = E.clone()
+        pot(phi)
+        got_phi = phi.clone()
+        assert np.array_equal(got_E.cpu().numpy().ravel(), np.ravel(want[0]))
+        assert np.array_equal(got_phi.cpu().numpy(), np.ravel(want[1]))
