@@ -200,24 +200,22 @@ void Engine::sort_items(const Layout& L, std::vector<int4>& items, bool field) c
     int4& it = items[i];
     it.w = 0;
     const SysDev& d = L.sd[it.x];
-    const int ncr = field ? d.fncr : d.ncr, chunk = field ? d.fchunk : d.chunk;
-    const int chunk_s = field ? d.fchunk_s : d.chunk_s;
-    const bool rk = it.z < 2 * ncr;
-    const int cb = it.z < ncr ? it.z : it.z - ncr;
+    const bool rk = it.z < d.ncr + d.nck;
+    const int cb = it.z < d.ncr ? it.z : it.z - d.ncr;
     int64_t nt, ns_, w = 10;
     if (sym && !field && rk) {
       // a real/Kelvin block against a chunk: both ways off the diagonal, one way on it (with
       // the self box checked)
-      nt = std::min<int64_t>(chunk, d.n - (int64_t)it.y * chunk);
+      nt = std::min<int64_t>(d.chunk, d.n - (int64_t)it.y * d.chunk);
       w = 12;
     } else {
       const int64_t tbk = field ? L.TBf : d.tb;
       nt = std::min<int64_t>(tbk, d.n - (int64_t)it.y * tbk);
     }
     if (rk) {
-      ns_ = std::min<int64_t>(chunk, d.n - (int64_t)cb * chunk);
+      ns_ = std::min<int64_t>(d.chunk, d.n - (int64_t)cb * d.chunk);
     } else {
-      ns_ = std::min<int64_t>(chunk_s, d.M - (int64_t)(it.z - 2 * ncr) * chunk_s);
+      ns_ = std::min<int64_t>(d.chunk_s, d.M - (int64_t)(it.z - d.ncr - d.nck) * d.chunk_s);
       w = 13;
     }
     keys[i] = Keyed{nt * ns_ * w, rk && !field ? std::abs(cb - it.y) : 0, (int)i};
@@ -232,13 +230,10 @@ void Engine::sort_items(const Layout& L, std::vector<int4>& items, bool field) c
 }
 
 // The real/Kelvin items to the front, in order; their number.
-int Engine::split_items(const Layout& L, std::vector<int4>& items, bool field) const
+int Engine::split_items(const Layout& L, std::vector<int4>& items) const
 {
   return (int)(std::stable_partition(items.begin(), items.end(),
-                                     [&](const int4& it) {
-                                       const SysDev& d = L.sd[it.x];
-                                       return it.z < 2 * (field ? d.fncr : d.ncr);
-                                     }) -
+                                     [&](const int4& it) { return it.z < L.sd[it.x].ncr + L.sd[it.x].nck; }) -
                items.begin());
 }
 
@@ -254,14 +249,14 @@ int Engine::make_field_items()
     L.it4f.reserve(L.n4f);
     for (int s = 0; s < (int)L.sd.size() && !L.tree; ++s) {
       const SysDev& d = L.sd[s];
-      const int nch = 2 * d.fncr + d.fncs, ntb = (d.n + L.TBf - 1) / L.TBf;
+      const int nch = d.ncr + d.nck + d.ncs, ntb = (d.n + L.TBf - 1) / L.TBf;
       for (int tb = 0; tb < ntb; ++tb)
         for (int c = 0; c < nch; ++c) L.it4f.push_back(make_int4(s, tb, c, 0));
     }
   }
   sort_items(L, L.it4f, true);
   L.it4fx = L.it4f;
-  L.nRKf = split_items(L, L.it4fx, true);
+  L.nRKf = split_items(L, L.it4fx);
   if (!L.it4f.empty()) {
     CK(cudaMemcpyAsync(it4f_d, L.it4f.data(), sizeof(int4) * L.it4f.size(), cudaMemcpyHostToDevice, stream));
     CK(cudaMemcpyAsync(it4fx_d, L.it4fx.data(), sizeof(int4) * L.it4fx.size(), cudaMemcpyHostToDevice, stream));
@@ -278,9 +273,6 @@ int Engine::make_field_items()
 //   share 0: 14.1 11.9 8.1 10.6;  1/8: 13.2 11.2 7.3 9.9;  1/4: 13.1 11.1 7.3 9.8;
 //   1/2: 13.4 11.5 7.2 10.0;  1: 13.8 11.5 7.6 10.2 (more partials and staging per pair)
 constexpr double kAloneShare = 0.25;
-
-// Bytes of field partials above which a layout's field chunks are merged (half of the L2).
-constexpr double kFieldMergeBytes = 64e6;
 
 // sizes_only: the workspace plan alone (the pair items are counted, not listed).
 Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_only) const
@@ -340,7 +332,6 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_o
   int64_t zoff = 0;
   int64_t chg = 0, surf = 0, coef = 0, mn = 0, mom = 0, part = 0, boxes = 0;
   int k5 = 0;
-  size_t nfield = 0;  // field items, one per chunk of the pair pass
   L.maxP = 1;
   L.pmax = 0;
   for (int s = 0; s < nsys; ++s) {
@@ -456,7 +447,7 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_o
           for (int c = d.ncr + d.nck; c < nch; ++c) L.it4.push_back(make_int4(s, tb, c, 0));
       }
       // the field kernel: every (target block, chunk) one way (no field pass with the tree)
-      if (!L.tree) nfield += (size_t)((n + TBf - 1) / TBf) * nch;
+      if (!L.tree) L.n4f += (size_t)((n + TBf - 1) / TBf) * nch;
     }
     chg += n;
     surf += sp.M;
@@ -506,25 +497,13 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_o
         for (int b = 0; b < (spec[s].M + pts - 1) / pts; ++b) L.it3m.push_back(make_int2(s, b));
     }
   }
-  // field chunks: two chunks of the pair pass each where that leaves four to eight items per CTA slot
-  // (see k_field.cu); the list itself is made by the first field pass (make_field_items)
   L.TBf = TBf;
-  const size_t fslots = (size_t)num_sms * std::max(prec == HSMA_FP64 ? occ_field64 : occ_field[cfg], 1);
-  const bool merges = prec != HSMA_FP64 && 32.0 * (double)part > kFieldMergeBytes;
-  const int merge = merges && nfield >= 8 * fslots && nfield < 16 * fslots ? 2 : 1;
-  for (auto& d : L.sd) {
-    d.fchunk = (int)std::min<int64_t>((int64_t)d.chunk * merge, std::max(d.chunk, d.n));
-    d.fchunk_s = (int)std::min<int64_t>((int64_t)d.chunk_s * merge, std::max(d.chunk_s, d.M));
-    d.fncr = (d.ncr + merge - 1) / merge;
-    d.fncs = (d.ncs + merge - 1) / merge;
-    if (!L.tree && prec != HSMA_FP64) L.n4f += (size_t)((d.n + TBf - 1) / TBf) * (2 * d.fncr + d.fncs);
-  }
   if (prec == HSMA_FP64) L.n4f = L.n4;
   if (!sizes_only) sort_items(L, L.it4, false);
   // the overlapped pass launches the real/Kelvin items (which need only the records) apart from
   // the surface items (which wait for the coefficient chain)
   L.it4x = L.it4;
-  if (!sizes_only) L.nRK = split_items(L, L.it4x, false);
+  if (!sizes_only) L.nRK = split_items(L, L.it4x);
   {
     // a sort block's share: all of a one-block system, else twice the mean share of its blocks
     // (a denser run of cells spills to the scratch buffer)

@@ -83,7 +83,7 @@ class Engine {
   int init(int dev, void* user_stream, int precision);
   Layout make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_only = false) const;
   void sort_items(const Layout& L, std::vector<int4>& items, bool field) const;
-  int split_items(const Layout& L, std::vector<int4>& items, bool field) const;
+  int split_items(const Layout& L, std::vector<int4>& items) const;
   int make_field_items();
   int set_sizes(const std::vector<int64_t>& ns);
   int attach(void* ptr, size_t bytes);

@@ -3,15 +3,10 @@
 // and dipole layers of the auxiliary sphere; Sec. 2.4, eqs. phicorrfinall and phirffinall),
 // differentiated term by term with the sources fixed, so that F_i = q_i E(x_i).
 //
-// Spatial order and the near/far box test are those of the potential pass.  A source chunk is one
-// chunk of the potential pass, or two where the partials would not stay in L2 and four to eight items
-// per CTA slot are left (SysDev::fchunk): every chunk costs a target 32 bytes of partials to write and
-// to reduce, and longer items end less evenly.  Fields and potentials, M = 2000, with one chunk and
-// with two: N = 13001 325 and 313 us, N = 20000 527 and 509 (608 and 602 for other charges),
-// N = 25000 860 and 882, N = 40000 1945 and 1985: merged up to about 20000.  Per (chunk, target)
-// the FP32 kernel writes two float4, the (hi, lo) two-sum pairs of (phi, Ex, Ey, Ez); the FP64 kernel
-// one (phi, Ex, Ey, Ez) in double.  k_reduce_field sums them in a fixed order (double-float on the
-// FP32 path) and maps them back to input order.
+// Work items, chunking, spatial order and the near/far box test are those of the potential
+// pass.  Per (chunk, target) the FP32 kernel writes two float4, the (hi, lo) two-sum pairs of
+// (phi, Ex, Ey, Ez); the FP64 kernel one (phi, Ex, Ey, Ez) in double.  k_reduce_field sums
+// them in a fixed order (double-float on the FP32 path) and maps them back to input order.
 //   point source Q at s:   phi += Q/d,  E += Q (t - s)/d^3
 //   surface point y (FP32, the dy -> 0 limit of the dipole pair, Dp = -D/R_tau):
 //     phi += (Q0 + Dp u)/d,  u = ((t - y).y)/d^2,
@@ -38,20 +33,20 @@ struct FChunk {
 __device__ __forceinline__ FChunk field_chunk(const SysDev& S, int c)
 {
   FChunk ci;
-  if (c < S.fncr) {
+  if (c < S.ncr) {
     ci.type = 0;
-    ci.first = c * S.fchunk;
-    ci.count = min(S.fchunk, S.n - ci.first);
+    ci.first = c * S.chunk;
+    ci.count = min(S.chunk, S.n - ci.first);
     ci.off = S.src + ci.first;
-  } else if (c < 2 * S.fncr) {
+  } else if (c < S.ncr + S.nck) {
     ci.type = 1;
-    ci.first = (c - S.fncr) * S.fchunk;
-    ci.count = min(S.fchunk, S.n - ci.first);
+    ci.first = (c - S.ncr) * S.chunk;
+    ci.count = min(S.chunk, S.n - ci.first);
     ci.off = S.src + S.n + ci.first;
   } else {
     ci.type = 2;
-    ci.first = (c - 2 * S.fncr) * S.fchunk_s;
-    ci.count = min(S.fchunk_s, S.M - ci.first);
+    ci.first = (c - S.ncr - S.nck) * S.chunk_s;
+    ci.count = min(S.chunk_s, S.M - ci.first);
     ci.off = S.surf + ci.first;
   }
   return ci;
@@ -545,14 +540,14 @@ __global__ __launch_bounds__(kFRedThreads) void k_reduce_field(
   const int n = S.n;
   const int sub = threadIdx.x % kFRedLanes;
   const int i = it.y * kFRedTargets + threadIdx.x / kFRedLanes;
-  const int nch = 2 * S.fncr + S.fncs;
+  const int nch = S.ncr + S.nck + S.ncs;
   double c[4] = {0.0, 0.0, 0.0, 0.0}, r[4] = {0.0, 0.0, 0.0, 0.0};
   if (prec == HSMA_FP64) {
     if (i < n) {
       const dbl4* b = fpart64 + S.part + i;
       for (int k = sub; k < nch; k += kFRedLanes) {
         const dbl4 v = b[(long long)k * n];
-        double* a = k < S.fncr ? c : r;
+        double* a = k < S.ncr ? c : r;
         a[0] += v.x;
         a[1] += v.y;
         a[2] += v.z;
@@ -571,8 +566,8 @@ __global__ __launch_bounds__(kFRedThreads) void k_reduce_field(
     for (int m = 0; m < 4; ++m) cc[m] = rr[m] = df_make(0.f, 0.f);
     if (i < n) {
       const float4* b = fpart + 2 * (S.part + i);
-      sum_field_chunks(b, n, sub, S.fncr, cc);
-      sum_field_chunks(b, n, S.fncr + sub, nch, rr);
+      sum_field_chunks(b, n, sub, S.ncr, cc);
+      sum_field_chunks(b, n, S.ncr + sub, nch, rr);
     }
     for (int o = 1; o < kFRedLanes; o <<= 1)
 #pragma unroll
