@@ -135,3 +135,32 @@ def test_fp32_potentials_scale_with_lengths_and_charges(threads, k, length, char
         b.hsma_batch_build_sources(np.array([300]), s * xyz, t * q)
         phi.append(b.hsma_batch_potential(api.HSMA_REACTION) * s / t)
     assert np.linalg.norm(phi[1] - phi[0]) <= 1e-6 * np.linalg.norm(phi[0])
+
+
+def _with_tiles(s, tiles, evaluate):
+    b = batch.from_systems([s])
+    b.hsma_batch_set_pair_config([tuple(c) for c in batch.pair_configs()].index(tiles))
+    b.hsma_batch_build_sources(np.array([s.n]), s.xyz, s.q)
+    return evaluate(b)
+
+
+TILES = [(128, 1, 4), (64, 2, 4), (64, 4, 8)]  # by work: below 6e6, below 1.2e8, above
+
+
+@pytest.mark.parametrize("line, n", [(6.0e6, 1437), (1.2e8, 7427)])
+def test_tile_rule_on_both_sides_of_its_lines(line, n):
+    """The untuned choice by the work N (2 N + 1.3 M), M = 1000, for the last size below a line and the
+    first above it: the potentials are those of that configuration to the bit, not those of the
+    neighbour's, and within 1e-6 of the oracle (the FP32 path's bound)."""
+    assert n * (2.0 * n + 1300.0) < line <= (n + 1) * (2.0 * n + 1302.0)
+    below = 0 if line == 6.0e6 else 1
+    for size, mine, other in ((n, TILES[below], TILES[below + 1]), (n + 1, TILES[below + 1], TILES[below])):
+        rng = np.random.default_rng(190880 + size)
+        s = inputs.System(1.0, 2.0, 80.0, 1.5, 12, 1000, inputs.uniform_ball(rng, size, 1.0), rng.choice([-1.0, 1.0], size))
+        h = api.hsma_create(s.a, s.eps1, s.eps2, s.kappa, api.hsma_default_params(p=s.p, M=s.M))
+        api.hsma_build_sources(h, s.xyz, s.q)
+        phi = api.hsma_potential(h)
+        assert np.array_equal(phi, _with_tiles(s, mine, lambda b: b.hsma_batch_potential()))
+        assert not np.array_equal(phi, _with_tiles(s, other, lambda b: b.hsma_batch_potential()))
+        ref = oracle.hsma(oracle.make_params(a=1.0, eps1=2.0, eps2=80.0, kappa=1.5, p=12, M=1000), s.xyz, s.q)["phi"]
+        assert np.linalg.norm(phi - ref) <= 1e-6 * np.linalg.norm(ref)
