@@ -76,7 +76,7 @@ int Engine::autotune(int reps, int* best_out, float* best_ms_out)
   reps = std::max(1, reps);
   const std::vector<int64_t> ns = cur_ns;
   size_t need = 0;
-  for (int c = 0; c < pair_config_count(); ++c) need = std::max(need, make_layout(ns, c, true).bytes);
+  for (int c = 0; c < pair_config_count(); ++c) need = std::max(need, make_layout(ns, c, c, true).bytes);
   if (need > ws_cap && ws_user) return fail(HSMA_E_OOM, "attached workspace too small to autotune");
   if (need > ws_cap) {
     // grow, keeping the inputs (at the same offsets in every layout)
@@ -244,10 +244,11 @@ int hsma_batch_workspace_size(hsma_batch_t* b, const int64_t* n, size_t* bytes)
   if (!sizes_ok(b, n, &tot)) return berr(b, HSMA_E_INVALID_ARG, "bad sizes");
   std::vector<int64_t> ns(n, n + b->e->spec.size());
   // the largest layout over all tile configurations, so that a workspace of this size also
-  // serves the autotuner
-  size_t mx = 0;
-  const int ncfg = b->e->prec == HSMA_FP64 ? 1 : hsma::pair_config_count();
-  for (int c = 0; c < ncfg; ++c) mx = std::max(mx, b->e->make_layout(ns, c, true).bytes);
+  // serves the autotuner, and the untuned one (whose field pass may have its own)
+  const bool f64 = b->e->prec == HSMA_FP64;
+  size_t mx = b->e->make_layout(ns, f64 ? 0 : b->e->choose_config(ns), f64 ? 0 : b->e->choose_field_config(ns), true).bytes;
+  for (int c = 0; c < (f64 ? 0 : hsma::pair_config_count()); ++c)
+    mx = std::max(mx, b->e->make_layout(ns, c, c, true).bytes);
   *bytes = mx;
   return HSMA_OK;
 }

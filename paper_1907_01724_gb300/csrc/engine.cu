@@ -200,22 +200,24 @@ void Engine::sort_items(const Layout& L, std::vector<int4>& items, bool field) c
     int4& it = items[i];
     it.w = 0;
     const SysDev& d = L.sd[it.x];
-    const bool rk = it.z < d.ncr + d.nck;
-    const int cb = it.z < d.ncr ? it.z : it.z - d.ncr;
+    const int ncr = field ? d.fncr : d.ncr, chunk = field ? d.fchunk : d.chunk;
+    const int chunk_s = field ? d.fchunk_s : d.chunk_s;
+    const bool rk = it.z < 2 * ncr;
+    const int cb = it.z < ncr ? it.z : it.z - ncr;
     int64_t nt, ns_, w = 10;
     if (sym && !field && rk) {
       // a real/Kelvin block against a chunk: both ways off the diagonal, one way on it (with
       // the self box checked)
-      nt = std::min<int64_t>(d.chunk, d.n - (int64_t)it.y * d.chunk);
+      nt = std::min<int64_t>(chunk, d.n - (int64_t)it.y * chunk);
       w = 12;
     } else {
       const int64_t tbk = field ? L.TBf : d.tb;
       nt = std::min<int64_t>(tbk, d.n - (int64_t)it.y * tbk);
     }
     if (rk) {
-      ns_ = std::min<int64_t>(d.chunk, d.n - (int64_t)cb * d.chunk);
+      ns_ = std::min<int64_t>(chunk, d.n - (int64_t)cb * chunk);
     } else {
-      ns_ = std::min<int64_t>(d.chunk_s, d.M - (int64_t)(it.z - d.ncr - d.nck) * d.chunk_s);
+      ns_ = std::min<int64_t>(chunk_s, d.M - (int64_t)(it.z - 2 * ncr) * chunk_s);
       w = 13;
     }
     keys[i] = Keyed{nt * ns_ * w, rk && !field ? std::abs(cb - it.y) : 0, (int)i};
@@ -230,10 +232,13 @@ void Engine::sort_items(const Layout& L, std::vector<int4>& items, bool field) c
 }
 
 // The real/Kelvin items to the front, in order; their number.
-int Engine::split_items(const Layout& L, std::vector<int4>& items) const
+int Engine::split_items(const Layout& L, std::vector<int4>& items, bool field) const
 {
   return (int)(std::stable_partition(items.begin(), items.end(),
-                                     [&](const int4& it) { return it.z < L.sd[it.x].ncr + L.sd[it.x].nck; }) -
+                                     [&](const int4& it) {
+                                       const SysDev& d = L.sd[it.x];
+                                       return it.z < 2 * (field ? d.fncr : d.ncr);
+                                     }) -
                items.begin());
 }
 
@@ -249,14 +254,14 @@ int Engine::make_field_items()
     L.it4f.reserve(L.n4f);
     for (int s = 0; s < (int)L.sd.size() && !L.tree; ++s) {
       const SysDev& d = L.sd[s];
-      const int nch = d.ncr + d.nck + d.ncs, ntb = (d.n + L.TBf - 1) / L.TBf;
+      const int nch = 2 * d.fncr + d.fncs, ntb = (d.n + L.TBf - 1) / L.TBf;
       for (int tb = 0; tb < ntb; ++tb)
         for (int c = 0; c < nch; ++c) L.it4f.push_back(make_int4(s, tb, c, 0));
     }
   }
   sort_items(L, L.it4f, true);
   L.it4fx = L.it4f;
-  L.nRKf = split_items(L, L.it4fx);
+  L.nRKf = split_items(L, L.it4fx, true);
   if (!L.it4f.empty()) {
     CK(cudaMemcpyAsync(it4f_d, L.it4f.data(), sizeof(int4) * L.it4f.size(), cudaMemcpyHostToDevice, stream));
     CK(cudaMemcpyAsync(it4fx_d, L.it4fx.data(), sizeof(int4) * L.it4fx.size(), cudaMemcpyHostToDevice, stream));
@@ -274,12 +279,45 @@ int Engine::make_field_items()
 //   1/2: 13.4 11.5 7.2 10.0;  1: 13.8 11.5 7.6 10.2 (more partials and staging per pair)
 constexpr double kAloneShare = 0.25;
 
+// Points per surface chunk for about `items` items of (a group of TB targets, a chunk): whole
+// 32-point boxes.
+static int surface_chunk(int64_t n, int M, int TB, double items)
+{
+  const int64_t n_tb = (n + TB - 1) / TB;
+  const int64_t want = std::max<int64_t>(1, std::llround(std::max(1.0, items) / n_tb));
+  return (int)std::max<int64_t>(kBox, ((M + want - 1) / want + kBox - 1) / kBox * kBox);
+}
+
+// Source chunks of n charges and M surface points on the FP32 path for about `items` pair items of a
+// tile configuration with groups of TB targets.
+struct Chunking {
+  int chunk, chunk_s, ncr, ncs;
+};
+static Chunking chunks_f32(int64_t n, int M, int TB, double items)
+{
+  Chunking c;
+  // real and Kelvin: nb blocks that are also the chunks, nb (nb + 1) items (each unordered
+  // pair of blocks once, real and Kelvin); a block is a whole number of the pair kernel's
+  // target groups and at most kSymChunkMax charges
+  const double items_rk = items * (2.0 * n) / (2.0 * n + 1.3 * M);
+  const int64_t nb = std::max<int64_t>(1, (int64_t)std::floor(std::sqrt(std::max(items_rk, 1.0))));
+  int64_t chunk = (n + nb - 1) / nb;
+  chunk = (chunk + TB - 1) / TB * TB;
+  chunk = std::min<int64_t>(std::max<int64_t>(chunk, TB), kSymChunkMax / TB * TB);
+  c.chunk = (int)chunk;
+  c.ncr = (int)((n + chunk - 1) / chunk);
+  c.chunk_s = surface_chunk(n, M, TB, items - items_rk);
+  c.ncs = (M + c.chunk_s - 1) / c.chunk_s;
+  return c;
+}
+
 // sizes_only: the workspace plan alone (the pair items are counted, not listed).
-Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_only) const
+Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, int fcfg, bool sizes_only) const
 {
   Layout L;
   const int nsys = (int)spec.size();
   L.cfg = cfg;
+  L.fcfg = fcfg;
   // TB: targets per pair item (FP64) or per surface item of the FP32 pair kernel (a warp's
   // group); TBf: targets per item of the FP32 field kernel (its CTA's targets)
   int TB, TBf, occ, nw;
@@ -290,14 +328,17 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_o
   } else {
     const PairConfig pc = pair_config(cfg);
     TB = 32 * pc.k;
-    TBf = pc.threads * pc.k;
+    TBf = pair_config(fcfg).threads * pair_config(fcfg).k;
     occ = occ_f32[cfg] > 0 ? occ_f32[cfg] : 1;
     nw = pair_workers_per_cta(cfg);
   }
   const int slots = num_sms * occ;
   // pair items wanted over the whole engine: a few per worker (CTA on the FP64 path, warp on the
   // FP32 path)
-  const double desired = (prec == HSMA_FP64 ? 4.0 : (double)pair_config(cfg).items_per_slot) * slots * nw;
+  auto desired_of = [&](int c) {
+    return (double)pair_config(c).items_per_slot * num_sms * std::max(occ_f32[c], 1) * pair_workers_per_cta(c);
+  };
+  const double desired = prec == HSMA_FP64 ? 4.0 * slots * nw : desired_of(cfg);
   // the pair items and moment blocks of the whole engine are apportioned by each system's share
   // of the work, so a batch of many small systems gets few, larger items per system
   double W = 0.0;
@@ -330,7 +371,7 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_o
   }
   L.sd.resize(nsys);
   int64_t zoff = 0;
-  int64_t chg = 0, surf = 0, coef = 0, mn = 0, mom = 0, part = 0, boxes = 0;
+  int64_t chg = 0, surf = 0, coef = 0, mn = 0, mom = 0, part = 0, fpart = 0, boxes = 0;
   int k5 = 0;
   L.maxP = 1;
   L.pmax = 0;
@@ -382,33 +423,36 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_o
         d.nck = d.ncr;
         d.ncs = (int)((sp.M + chunk - 1) / chunk);
       } else {
-        // real and Kelvin: nb blocks that are also the chunks, nb (nb + 1) items (each unordered
-        // pair of blocks once, real and Kelvin); a block is a whole number of the pair kernel's
-        // target groups and at most kSymChunkMax charges
-        const double items_rk = L.tree ? 0.0 : items_s * (2.0 * n) / (2.0 * n + 1.3 * sp.M);
+        Chunking c = chunks_f32(n, sp.M, TB, items_s);
         if (L.tree) {
-          // kTreeRootSplit chunks each: the tree's real and Kelvin sums (k_tree_eval), no pair items
-          d.chunk = (int)n;
-          d.ncr = d.nck = kTreeRootSplit;
-        } else {
-          const int64_t nb = std::max<int64_t>(1, (int64_t)std::floor(std::sqrt(std::max(items_rk, 1.0))));
-          int64_t chunk = (n + nb - 1) / nb;
-          chunk = (chunk + TB - 1) / TB * TB;
-          chunk = std::min<int64_t>(std::max<int64_t>(chunk, TB), kSymChunkMax / TB * TB);
-          d.chunk = (int)chunk;
-          d.ncr = (int)((n + chunk - 1) / chunk);
-          d.nck = d.ncr;
+          // kTreeRootSplit chunks each: the tree's real and Kelvin sums (k_tree_eval), no pair
+          // items, and all of the items for the surface
+          c.chunk = (int)n;
+          c.ncr = kTreeRootSplit;
+          c.chunk_s = surface_chunk(n, sp.M, TB, items_s);
+          c.ncs = (sp.M + c.chunk_s - 1) / c.chunk_s;
         }
-        // surface: the rest of the items over the target groups, chunks of whole 32-point boxes
-        const double items_sf = std::max(1.0, items_s - items_rk);
-        const int64_t ncs_want = std::max<int64_t>(1, std::llround(items_sf / d.n_tb));
-        int64_t chunk_s = (sp.M + ncs_want - 1) / ncs_want;
-        chunk_s = std::max<int64_t>(kBox, (chunk_s + kBox - 1) / kBox * kBox);
-        d.chunk_s = (int)chunk_s;
-        d.ncs = (int)((sp.M + chunk_s - 1) / chunk_s);
+        d.chunk = c.chunk;
+        d.ncr = d.nck = c.ncr;
+        d.chunk_s = c.chunk_s;
+        d.ncs = c.ncs;
+        // the field pass: by its own configuration (choose_field_config)
+        const Chunking f = fcfg == cfg ? c : chunks_f32(n, sp.M, 32 * pair_config(fcfg).k, std::max(1.0, std::round(
+                                                           desired_of(fcfg) * share)));
+        d.fchunk = f.chunk;
+        d.fncr = f.ncr;
+        d.fchunk_s = f.chunk_s;
+        d.fncs = f.ncs;
+      }
+      if (prec == HSMA_FP64) {
+        d.fchunk = d.chunk;
+        d.fncr = d.ncr;
+        d.fchunk_s = d.chunk_s;
+        d.fncs = d.ncs;
       }
     }
     d.part = part;
+    d.fpart = fpart;
     d.dc2 = (float)((kNearRel * sp.a) * (kNearRel * sp.a));
     d.bb = boxes;
     d.k5_first = k5;
@@ -447,7 +491,7 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_o
           for (int c = d.ncr + d.nck; c < nch; ++c) L.it4.push_back(make_int4(s, tb, c, 0));
       }
       // the field kernel: every (target block, chunk) one way (no field pass with the tree)
-      if (!L.tree) L.n4f += (size_t)((n + TBf - 1) / TBf) * nch;
+      if (!L.tree) L.n4f += (size_t)((n + TBf - 1) / TBf) * (2 * d.fncr + d.fncs);
     }
     chg += n;
     surf += sp.M;
@@ -455,6 +499,7 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_o
     mn += sp.p + 1;
     mom += d.mom_blocks;
     part += (int64_t)nch * n;
+    fpart += (int64_t)(2 * d.fncr + d.fncs) * n;
     boxes += 2 * ((n + kBox - 1) / kBox);
     k5 += d.k5_count;
     L.maxP = std::max(L.maxP, d.P);
@@ -503,7 +548,7 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_o
   // the overlapped pass launches the real/Kelvin items (which need only the records) apart from
   // the surface items (which wait for the coefficient chain)
   L.it4x = L.it4;
-  if (!sizes_only) L.nRK = split_items(L, L.it4x);
+  if (!sizes_only) L.nRK = split_items(L, L.it4x, false);
   {
     // a sort block's share: all of a one-block system, else twice the mean share of its blocks
     // (a denser run of cells spills to the scratch buffer)
@@ -519,6 +564,7 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_o
   L.totMom = mom;
   L.totZ = zoff;
   L.totPart = part;
+  L.totFpart = fpart;
   L.totBoxes = boxes;
   L.mom_stride = (int)align_up((size_t)L.maxP + 1, 2);
   L.nw = nw;
@@ -754,7 +800,7 @@ int Engine::set_sizes(const std::vector<int64_t>& ns)
 {
   if (have_layout && ns == cur_ns && layout_uploaded) return HSMA_OK;
   const int cfg = prec == HSMA_FP64 ? 0 : choose_config(ns);
-  L = make_layout(ns, cfg);
+  L = make_layout(ns, cfg, prec == HSMA_FP64 ? 0 : choose_field_config(ns));
   rk_side = prec == HSMA_FP64 ? 1 : choose_side(ns);
   cur_ns = ns;
   have_layout = true;
@@ -1300,7 +1346,7 @@ int Engine::ensure_host_stage(int64_t count)
 
 int Engine::ensure_field_buffers()
 {
-  const size_t need_p = std::max<size_t>(32 * (size_t)L.totPart, 256);
+  const size_t need_p = std::max<size_t>(32 * (size_t)L.totFpart, 256);
   const size_t need_e = std::max<size_t>(72 * (size_t)L.totN, 256);
   if (need_p <= fpart_cap && need_e <= E_cap) {
     Ec_d = E_d;
@@ -1344,7 +1390,7 @@ int Engine::ensure_field_buffers()
 
 int Engine::field_slots() const
 {
-  return num_sms * std::max(prec == HSMA_FP64 ? occ_field64 : occ_field[L.cfg], 1);
+  return num_sms * std::max(prec == HSMA_FP64 ? occ_field64 : occ_field[L.fcfg], 1);
 }
 
 void Engine::launch_field_items(PairWork w1, PairWork w2, int grid, cudaStream_t st, bool pdl)
@@ -1353,7 +1399,7 @@ void Engine::launch_field_items(PairWork w1, PairWork w2, int grid, cudaStream_t
   if (prec == HSMA_FP64)
     launch_field_f64(grid, sys_d, w1, w2, src64_d, surf64a_d, surf64b_d, (dbl4*)fpart_d, st, pdl);
   else
-    launch_field_f32(L.cfg, grid, sys_d, w1, w2, srchi_d, srclo_d, surfa_d, surfb_d, boxes_d, (float4*)fpart_d, st,
+    launch_field_f32(L.fcfg, grid, sys_d, w1, w2, srchi_d, srclo_d, surfa_d, surfb_d, boxes_d, (float4*)fpart_d, st,
                      pdl);
 }
 
@@ -1550,6 +1596,17 @@ static int config_of(int threads, int k, int items_per_slot)
   return 0;
 }
 
+// The autotuned choice cached for the size bucket of a set of sizes, or null.
+const Engine::Tuned* Engine::tuned_entry(const std::vector<int64_t>& ns) const
+{
+  int64_t tot = 0;
+  for (auto v : ns) tot += v;
+  const int bucket = tune_bucket(tot, (int)ns.size());
+  for (const auto& e : tuned)
+    if (e.bucket == bucket) return &e;
+  return nullptr;
+}
+
 // Pair-sum tile configuration for a set of sizes: the autotuned choice if one is cached for
 // this size bucket, else by the pair work W = sum N (2N + 1.3 M) of the engine: groups of 32 K
 // targets, small while there are fewer items than warps (a launch is then as long as its longest
@@ -1566,17 +1623,26 @@ static int config_of(int threads, int k, int items_per_slot)
 int Engine::choose_config(const std::vector<int64_t>& ns) const
 {
   if (forced_cfg >= 0) return forced_cfg;
-  int64_t tot = 0;
   double W = 0.0;
-  for (size_t s = 0; s < ns.size(); ++s) {
-    tot += ns[s];
-    W += (double)ns[s] * (2.0 * (double)ns[s] + 1.3 * spec[s].M);
-  }
-  const int bucket = tune_bucket(tot, (int)ns.size());
-  for (const auto& e : tuned)
-    if (e.bucket == bucket) return e.cfg;
+  for (size_t s = 0; s < ns.size(); ++s) W += (double)ns[s] * (2.0 * (double)ns[s] + 1.3 * spec[s].M);
+  if (const Tuned* e = tuned_entry(ns)) return e->cfg;
   static const int small = config_of(128, 1, 4), medium = config_of(64, 2, 4), large = config_of(64, 4, 8);
   return W < 6.0e6 ? small : (W < 1.2e8 ? medium : large);
+}
+
+// Tile configuration of the field pass: a forced or autotuned one is the pair pass's; else by the same
+// work W the pair pass's smallest groups, and from there CTAs of 128 threads with 4 targets each.  The
+// pair pass's own choices serve the field worse: a chunk costs every target 32 bytes of partials, and
+// CTAs of 64 threads stage each source for half as many targets.  Field steps with the pair pass's
+// tiles and with these, in us, passes on several streams: N = 5000 68.1 and 61.5, 9000 145.2 and 142.7,
+// 13001 262 and 251, 16000 361 and 339, 20000 527 and 519, 40000 1772 and 1750; 64 x 1000 375 and 367.
+// (Alone on the GPU, where longer items end less evenly, the first are faster at some sizes: N = 9000
+// 170 and 178, 20000 586 and 606, 30000 1175 and 1192, but 13001 290 and 287, 16000 431 and 418.)
+int Engine::choose_field_config(const std::vector<int64_t>& ns) const
+{
+  const int cfg = choose_config(ns);
+  static const int small = config_of(128, 1, 4), field = config_of(128, 4, 4);
+  return forced_cfg >= 0 || tuned_entry(ns) || cfg == small ? cfg : field;
 }
 
 // Schedule of the real/Kelvin pair items in the fused graph: forced, else the size class's
@@ -1585,11 +1651,7 @@ int Engine::choose_config(const std::vector<int64_t>& ns) const
 int Engine::choose_side(const std::vector<int64_t>& ns) const
 {
   if (forced_side >= 0) return forced_side;
-  int64_t tot = 0;
-  for (auto v : ns) tot += v;
-  const int bucket = tune_bucket(tot, (int)ns.size());
-  for (const auto& e : tuned)
-    if (e.bucket == bucket) return e.side;
+  if (const Tuned* e = tuned_entry(ns)) return e->side;
   return ns.size() <= 8 ? 1 : 0;
 }
 
@@ -1757,8 +1819,8 @@ const char* hsma_last_error(const hsma_t* h)
 int hsma_workspace_size(hsma_t* h, int64_t n, size_t* bytes)
 {
   if (!h || !bytes || n < 0 || n > (int64_t)INT32_MAX / 4) return set_err(h, HSMA_E_INVALID_ARG, "bad argument");
-  const int cfg = h->e->prec == HSMA_FP64 ? 0 : h->e->choose_config({n});
-  *bytes = h->e->make_layout({n}, cfg, true).bytes;
+  const bool f64 = h->e->prec == HSMA_FP64;
+  *bytes = h->e->make_layout({n}, f64 ? 0 : h->e->choose_config({n}), f64 ? 0 : h->e->choose_field_config({n}), true).bytes;
   return HSMA_OK;
 }
 

@@ -51,10 +51,11 @@ struct Layout {
   std::vector<int2> selrng;   // their reduce-item ranges
   size_t o_sel = 0, o_selrng = 0;
   int cfg = 0, maxP = 1, pmax = 0, mom_stride = 3, pair_grid = 1;
+  int fcfg = 0;              // tile configuration of the field pass
   int TBf = 1;               // targets per field item
   size_t n4 = 0, n4f = 0;    // pair and field items
   bool field_items = false;  // it4f, it4fx made and uploaded
-  int64_t totN = 0, totM = 0, totP = 0, totMn = 0, totMom = 0, totPart = 0;
+  int64_t totN = 0, totM = 0, totP = 0, totMn = 0, totMom = 0, totPart = 0, totFpart = 0;
   size_t o_sys = 0, o_Mn = 0, o_rec_a = 0, o_rec_b = 0, o_sect = 0, o_inv_np1 = 0, o_xyz = 0, o_q = 0;
   size_t o_rec_a2 = 0, o_rec_b2 = 0, o_sect2 = 0, o_mtab = 0;
   size_t o_mgeo = 0, o_mz = 0, o_mwq = 0, o_mcen = 0, o_itmu = 0;
@@ -81,9 +82,9 @@ class Engine {
  public:
   ~Engine();
   int init(int dev, void* user_stream, int precision);
-  Layout make_layout(const std::vector<int64_t>& ns, int cfg, bool sizes_only = false) const;
+  Layout make_layout(const std::vector<int64_t>& ns, int cfg, int fcfg, bool sizes_only = false) const;
   void sort_items(const Layout& L, std::vector<int4>& items, bool field) const;
-  int split_items(const Layout& L, std::vector<int4>& items) const;
+  int split_items(const Layout& L, std::vector<int4>& items, bool field) const;
   int make_field_items();
   int set_sizes(const std::vector<int64_t>& ns);
   int attach(void* ptr, size_t bytes);
@@ -108,6 +109,7 @@ class Engine {
   int delta_energy(int64_t k, const double* x_new, double* de);
   int apply_move(int64_t k, const double* x_new);
   int choose_config(const std::vector<int64_t>& ns) const;
+  int choose_field_config(const std::vector<int64_t>& ns) const;
   int choose_side(const std::vector<int64_t>& ns) const;
   int autotune(int reps, int* best, float* best_ms);
   int tune_time_config(int c, int side, int steps, std::vector<float>& t);  // (autotune) steps after a rebuild
@@ -142,6 +144,7 @@ class Engine {
     int bucket, cfg, side;
   };
   std::vector<Tuned> tuned;  // autotuned choices per size class
+  const Tuned* tuned_entry(const std::vector<int64_t>& ns) const;
   std::vector<int> occ_f32, occ_field;
   std::vector<int> regs_f32;  // registers of a CTA of each FP32 pair configuration
   int chain_regs = 0;         // registers of the largest coefficient / surface CTA

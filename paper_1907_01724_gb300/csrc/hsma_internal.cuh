@@ -123,6 +123,9 @@ struct SysDev {
   int chunk;          // sources per real/Kelvin chunk; FP32 path: also the targets per block of
                       // the pair kernel's real/Kelvin items (blocks and chunks coincide)
   int chunk_s;        // points per surface chunk
+  int fncr, fncs;     // the field pass's source chunks: real (as many Kelvin) and surface ones, of
+  int fchunk, fchunk_s;  // fchunk charges and fchunk_s points
+  long long fpart;    // offset of its field partials (their chunks * n elements)
   int tb;             // targets per target block of the pair kernel's surface items (FP32 path:
                       // a warp's group, 32 K) and of every FP64 pair item
   int n_tb;           // such target blocks

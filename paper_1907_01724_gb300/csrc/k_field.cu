@@ -3,8 +3,8 @@
 // and dipole layers of the auxiliary sphere; Sec. 2.4, eqs. phicorrfinall and phirffinall),
 // differentiated term by term with the sources fixed, so that F_i = q_i E(x_i).
 //
-// Work items, chunking, spatial order and the near/far box test are those of the potential
-// pass.  Per (chunk, target) the FP32 kernel writes two float4, the (hi, lo) two-sum pairs of
+// Work items, spatial order and the near/far box test are those of the potential pass; the tiles (a
+// CTA's targets, the source chunks) are the field pass's own (Engine::choose_field_config).  Per (chunk, target) the FP32 kernel writes two float4, the (hi, lo) two-sum pairs of
 // (phi, Ex, Ey, Ez); the FP64 kernel one (phi, Ex, Ey, Ez) in double.  k_reduce_field sums
 // them in a fixed order (double-float on the FP32 path) and maps them back to input order.
 //   point source Q at s:   phi += Q/d,  E += Q (t - s)/d^3
@@ -33,20 +33,20 @@ struct FChunk {
 __device__ __forceinline__ FChunk field_chunk(const SysDev& S, int c)
 {
   FChunk ci;
-  if (c < S.ncr) {
+  if (c < S.fncr) {
     ci.type = 0;
-    ci.first = c * S.chunk;
-    ci.count = min(S.chunk, S.n - ci.first);
+    ci.first = c * S.fchunk;
+    ci.count = min(S.fchunk, S.n - ci.first);
     ci.off = S.src + ci.first;
-  } else if (c < S.ncr + S.nck) {
+  } else if (c < 2 * S.fncr) {
     ci.type = 1;
-    ci.first = (c - S.ncr) * S.chunk;
-    ci.count = min(S.chunk, S.n - ci.first);
+    ci.first = (c - S.fncr) * S.fchunk;
+    ci.count = min(S.fchunk, S.n - ci.first);
     ci.off = S.src + S.n + ci.first;
   } else {
     ci.type = 2;
-    ci.first = (c - S.ncr - S.nck) * S.chunk_s;
-    ci.count = min(S.chunk_s, S.M - ci.first);
+    ci.first = (c - 2 * S.fncr) * S.fchunk_s;
+    ci.count = min(S.fchunk_s, S.M - ci.first);
     ci.off = S.surf + ci.first;
   }
   return ci;
@@ -334,7 +334,7 @@ __global__ __launch_bounds__(NT) void k_field_f32(const SysDev* __restrict__ sys
       }
       __syncthreads();
     }
-    float4* out = fpart + 2 * (S.part + (long long)it.z * n);
+    float4* out = fpart + 2 * (S.fpart + (long long)it.z * n);
 #pragma unroll
     for (int k = 0; k < K; ++k)
       if (tix[k] < n) {
@@ -468,7 +468,7 @@ __global__ __launch_bounds__(kF64FThreads) void k_field_f64(const SysDev* __rest
       }
       __syncthreads();
     }
-    if (i < n) fpart64[S.part + (long long)it.z * n + i] = make_dbl4(ap, ax, ay, az);
+    if (i < n) fpart64[S.fpart + (long long)it.z * n + i] = make_dbl4(ap, ax, ay, az);
   }
 }
 
@@ -540,14 +540,14 @@ __global__ __launch_bounds__(kFRedThreads) void k_reduce_field(
   const int n = S.n;
   const int sub = threadIdx.x % kFRedLanes;
   const int i = it.y * kFRedTargets + threadIdx.x / kFRedLanes;
-  const int nch = S.ncr + S.nck + S.ncs;
+  const int nch = 2 * S.fncr + S.fncs;
   double c[4] = {0.0, 0.0, 0.0, 0.0}, r[4] = {0.0, 0.0, 0.0, 0.0};
   if (prec == HSMA_FP64) {
     if (i < n) {
-      const dbl4* b = fpart64 + S.part + i;
+      const dbl4* b = fpart64 + S.fpart + i;
       for (int k = sub; k < nch; k += kFRedLanes) {
         const dbl4 v = b[(long long)k * n];
-        double* a = k < S.ncr ? c : r;
+        double* a = k < S.fncr ? c : r;
         a[0] += v.x;
         a[1] += v.y;
         a[2] += v.z;
@@ -565,9 +565,9 @@ __global__ __launch_bounds__(kFRedThreads) void k_reduce_field(
 #pragma unroll
     for (int m = 0; m < 4; ++m) cc[m] = rr[m] = df_make(0.f, 0.f);
     if (i < n) {
-      const float4* b = fpart + 2 * (S.part + i);
-      sum_field_chunks(b, n, sub, S.ncr, cc);
-      sum_field_chunks(b, n, S.ncr + sub, nch, rr);
+      const float4* b = fpart + 2 * (S.fpart + i);
+      sum_field_chunks(b, n, sub, S.fncr, cc);
+      sum_field_chunks(b, n, S.fncr + sub, nch, rr);
     }
     for (int o = 1; o < kFRedLanes; o <<= 1)
 #pragma unroll

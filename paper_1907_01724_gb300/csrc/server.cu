@@ -720,7 +720,8 @@ int hsma_server_load(hsma_server_t* s, const int64_t* n, const double* xyz, cons
     // device footprint of the chain on its own
     Engine& e = *s->e;
     e.spec = {s->specs[c]};
-    s->footprint[c] = e.make_layout({n[c]}, e.prec == HSMA_FP64 ? 0 : e.choose_config({n[c]}), true).bytes;
+    const int cfg = e.prec == HSMA_FP64 ? 0 : e.choose_config({n[c]});
+    s->footprint[c] = e.make_layout({n[c]}, cfg, cfg, true).bytes;
     off += n[c];
   }
   int rc = admit(s, admitted);

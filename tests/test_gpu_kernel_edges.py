@@ -164,3 +164,27 @@ def test_tile_rule_on_both_sides_of_its_lines(line, n):
         assert not np.array_equal(phi, _with_tiles(s, other, lambda b: b.hsma_batch_potential()))
         ref = oracle.hsma(oracle.make_params(a=1.0, eps1=2.0, eps2=80.0, kappa=1.5, p=12, M=1000), s.xyz, s.q)["phi"]
         assert np.linalg.norm(phi - ref) <= 1e-6 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("n, tiles", [(300, (128, 1, 4)), (1437, (128, 1, 4)), (1438, (128, 4, 4)), (7428, (128, 4, 4)),
+                                      (20000, (128, 4, 4))])
+def test_field_pass_has_its_own_tiles(n, tiles):
+    """The untuned field pass, M = 1000: the pair pass's smallest tiles below a work N (2 N + 1.3 M) of
+    6e6, CTAs of 128 threads with 4 targets each above, whatever the pair pass takes there: fields and
+    the potentials of the same pass are those of that configuration to the bit, potentials of a later
+    pass again those of the pair pass, and the chunks cover every source (1e-6 of the FP64 field pass)."""
+    rng = np.random.default_rng(190890 + n)
+    s = inputs.System(1.0, 2.0, 80.0, 1.5, 12, 1000, inputs.uniform_ball(rng, n, 1.0), rng.choice([-1.0, 1.0], n))
+    out = {}
+    for prec in (api.HSMA_FP32, api.HSMA_FP64):
+        h = api.hsma_create(s.a, s.eps1, s.eps2, s.kappa, api.hsma_default_params(p=s.p, M=s.M, precision=prec))
+        api.hsma_build_sources(h, s.xyz, s.q)
+        pairs = api.hsma_potential(h)
+        api.hsma_build_sources(h, s.xyz, s.q)
+        out[prec] = [api.hsma_field(h).reshape(-1), api.hsma_potential(h)]
+        api.hsma_build_sources(h, s.xyz, s.q)
+        assert np.array_equal(api.hsma_potential(h), pairs)
+    want = _with_tiles(s, tiles, lambda b: [np.reshape(b.hsma_batch_field(), -1), b.hsma_batch_potential()])
+    for a, b, c in zip(out[api.HSMA_FP32], want, out[api.HSMA_FP64]):
+        assert np.array_equal(a, b)
+        assert np.linalg.norm(a - c) <= 1e-6 * np.linalg.norm(c)
