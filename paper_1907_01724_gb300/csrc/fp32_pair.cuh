@@ -15,17 +15,21 @@ __device__ __forceinline__ float rsqrt_mufu(float x)
   return y;
 }
 
-// 1/sqrt(x): the approximate reciprocal root (relative error below 2^-19), then, with e = 1 - x y^2,
-// y + y e (1/2 + 3/8 e) (the next term, 5/16 e^3, is below 2^-56).  Arguments whose exponent leaves
-// no room for the step (zero, subnormal, near overflow, not finite) take the square root and the
-// division.
+// 1/sqrt(x): the approximate reciprocal root y, then, with e = 1 - x y^2, the binomial series of
+// (1 - e)^(-1/2): y + y e (1/2 + 3/8 e).  y has 21 significant bits (the instruction leaves the low
+// word zero), so y^2 is exact and e, |e| <= 2^-19.04, has one rounding of 2^-72; the next term of the
+// series, 5/16 e^3, is below 2^-58.  So the error is the last operation's rounding: over
+// 2^28 arguments at most 1.016 x 2^-53, rms 0.433, as CUDA's rsqrt(); the root and the division that
+// it replaces 1.499 and 0.601, and the same step with e = 1 - (x y) y 1.257 and 0.481.
+// Arguments whose exponent leaves no room for the step (zero, subnormal, near overflow, not finite)
+// take the square root and the division.
 __device__ __forceinline__ double rsqrt_f64(double x)
 {
   const unsigned int top = (unsigned int)__double2hiint(x) >> 20;  // sign and exponent
   if (top - 0x040u > 0x780u - 0x040u) return 1.0 / sqrt(x);
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-(x * y), y, 1.0);
+  const double e = fma(-x, y * y, 1.0);
   return fma(y * e, fma(0.375, e, 0.5), y);
 }
 

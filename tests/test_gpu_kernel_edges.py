@@ -188,3 +188,26 @@ def test_field_pass_has_its_own_tiles(n, tiles):
     for a, b, c in zip(out[api.HSMA_FP32], want, out[api.HSMA_FP64]):
         assert np.array_equal(a, b)
         assert np.linalg.norm(a - c) <= 1e-6 * np.linalg.norm(c)
+
+
+def test_fp64_reciprocal_roots():
+    """The FP64 pair kernel's 1/d over random distances at many exponents, inside its fast range, at
+    both of its ends (d^2 = 2^-959 and 2^898) and in the fallback past them: 2048 cavities with a unit
+    charge at +d/2 and one at -d/2, whose Coulomb potentials are 1/d of d^2 = fl(d d) with no other
+    rounding.  In the fast range the last operation's rounding, 2^-53, and the terms left out, below
+    2^-58, are allowed; in the fallback those of a root and a division, 2^-52 together."""
+    rng = np.random.default_rng(190870)
+    exps = np.repeat([-505, -490, -481, -480, -479, -478, -300, -1, 0, 1, 300, 447, 448, 449, 450, 500], 128)
+    d = np.ldexp(rng.uniform(1.0, 2.0, exps.size), exps)
+    x = np.zeros((exps.size, 2, 3))
+    axis = np.arange(exps.size) % 3
+    x[np.arange(exps.size), 0, axis], x[np.arange(exps.size), 1, axis] = 0.5 * d, -0.5 * d
+    b = batch.Batch(d, np.ones_like(d), np.full_like(d, 2.0), np.zeros_like(d),
+                    api.hsma_default_params(p=2, M=4, coulomb_k=1.0, precision=api.HSMA_FP64))
+    b.hsma_batch_build_sources(np.full(exps.size, 2), x.reshape(-1, 3), np.ones(2 * exps.size))
+    phi = b.hsma_batch_potential(api.HSMA_COULOMB).reshape(-1, 2).astype(np.longdouble)
+    d2 = (d * d).astype(np.longdouble)[:, None]
+    err = np.abs(phi * phi * d2 - 1.0) / 2.0
+    fast = (d2 >= np.ldexp(np.longdouble(1.0), -959)) & (d2 < np.ldexp(np.longdouble(1.0), 898))
+    assert 0 < fast.sum() < fast.size
+    assert (err <= np.where(fast, 2.0 ** -53 + 2.0 ** -58, 2.0 ** -52)).all(), err.max() * 2.0 ** 53
