@@ -993,7 +993,7 @@ void Engine::issue_pot()
     const int nit = (int)L.it4.size();
     const PairWork all{it4_d, nit, ctr_pairs_d, std::min(L.pair_grid * L.nw, nit)}, none{nullptr, 0, nullptr, 0};
     if (prec == HSMA_FP64)
-      launch_pairs_f64(L.pair_grid, sys_d, all, none, src64_d, surf64a_d, surf64b_d, part64_d, stream);
+      launch_pairs_f64(wide_shells(), L.pair_grid, sys_d, all, none, src64_d, surf64a_d, surf64b_d, part64_d, stream);
     else
       launch_pairs_f32(L.cfg, L.pair_grid, sys_d, all, none, srchi_d, srclo_d, surfa_d, surfb_d, boxes_d, part_d,
                        stream);
@@ -1016,7 +1016,7 @@ void Engine::launch_pair_items(PairWork w1, PairWork w2, int grid, cudaStream_t 
 {
   if (w1.nitems <= 0 && w2.nitems <= 0) return;
   if (prec == HSMA_FP64)
-    launch_pairs_f64(grid, sys_d, w1, w2, src64_d, surf64a_d, surf64b_d, part64_d, st, pdl);
+    launch_pairs_f64(wide_shells(), grid, sys_d, w1, w2, src64_d, surf64a_d, surf64b_d, part64_d, st, pdl);
   else
     launch_pairs_f32(L.cfg, grid, sys_d, w1, w2, srchi_d, srclo_d, surfa_d, surfb_d, boxes_d, part_d, st, pdl);
 }
@@ -1594,6 +1594,16 @@ static int config_of(int threads, int k, int items_per_slot)
     if (p.threads == threads && p.k == k && p.items_per_slot == items_per_slot) return c;
   }
   return 0;
+}
+
+// Whether a system's dipole shells reach among its charges (dy > R_tau - a; see k_pairs_f64).
+bool Engine::wide_shells() const
+{
+  for (const auto& s : spec) {
+    const double Rtau = (1.0 + s.tau) * s.a;
+    if (s.dy_rel * Rtau > Rtau - s.a) return true;
+  }
+  return false;
 }
 
 // The autotuned choice cached for the size bucket of a set of sizes, or null.

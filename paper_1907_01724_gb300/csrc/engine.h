@@ -144,6 +144,7 @@ class Engine {
     int bucket, cfg, side;
   };
   std::vector<Tuned> tuned;  // autotuned choices per size class
+  bool wide_shells() const;
   const Tuned* tuned_entry(const std::vector<int64_t>& ns) const;
   std::vector<int> occ_f32, occ_field;
   std::vector<int> regs_f32;  // registers of a CTA of each FP32 pair configuration

@@ -299,7 +299,7 @@ constexpr int kReduceTargetsPerBlock = 32;
 void launch_pairs_f32(int cfg, int grid, const SysDev* sys, PairWork w1, PairWork w2, const float4* src_hi,
                       const float4* src_lo, const float4* surf_a, const float4* surf_b, const float4* boxes,
                       float2* part, cudaStream_t st, bool pdl = false);
-void launch_pairs_f64(int grid, const SysDev* sys, PairWork w1, PairWork w2, const dbl4* src64,
+void launch_pairs_f64(bool wide, int grid, const SysDev* sys, PairWork w1, PairWork w2, const dbl4* src64,
                       const dbl4* surf64_a, const double* surf64_b, double* part64, cudaStream_t st,
                       bool pdl = false);
 // Reduce the pair partials of the launched items to potentials and energies; the energies of

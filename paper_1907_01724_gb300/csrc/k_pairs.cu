@@ -146,12 +146,17 @@ void launch_pairs_f32(int cfg, int grid, const SysDev* sys, PairWork w1, PairWor
 //      2 B / (d_+ d_- (d_+ + d_-)) = 2 B / (s sqrt(2 A + 2 s)),  s = d_+ d_- = sqrt(A^2 - C^2)
 //    (two reciprocal roots, no division), and B = (R_tau^2 - |x|^2 + d0^2) / (2 R_tau), every term
 //    positive inside the cavity, needs no unit vector of the point.  A, B and C are taken in units
-//    of R_tau, so that A^2 stays in range for a cavity of any size.
+//    of R_tau, so that A^2 stays in range for a cavity of any size.  A^2 - C^2 loses the digits of
+//    A^2/(d_+ d_-)^2, at most 2.8 while dy <= R_tau - a; a wider dy puts the inner shell among the
+//    charges (d_- -> 0), and its points take the two distances themselves (WIDE, an instance of its
+//    own: in one kernel the two forms take 72 registers instead of 56, and a step of N = 1999 takes
+//    591 us instead of 498).
 // A step of N = 1999, M = 1000, p = 20 (one GB300): 1300 us with the square roots and divisions of
 // the plain definition (five roots and divisions and a unit vector per surface point), 500 us so,
 // at the same error against the 64-bit definition (1.2e-15).
 constexpr int kF64Threads = kF64TargetsPerBlock;
 
+template <bool WIDE>
 __global__ __launch_bounds__(kF64Threads) void k_pairs_f64(const SysDev* __restrict__ sys, PairWork w1,
                                                            PairWork w2, const dbl4* __restrict__ src64,
                                                            const dbl4* __restrict__ surf64_a,
@@ -194,7 +199,21 @@ __global__ __launch_bounds__(kF64Threads) void k_pairs_f64(const SysDev* __restr
         }
       }
       __syncthreads();
-      if (ch.type == 2) {
+      if (WIDE && ch.type == 2 && S.dy > S.Rtau - S.a) {
+        const double rm = 1.0 - 0.5 * dy, rp = 1.0 + 0.5 * dy;
+        const double tx = tg.x * S.inv_Rt, ty = tg.y * S.inv_Rt, tz = tg.z * S.inv_Rt;
+        for (int s = 0; s < cnt; ++s) {
+          const dbl4 y = shA[s];
+          const double dx = tg.x - y.x, dy_ = tg.y - y.y, dz = tg.z - y.z;
+          acc = fma(y.w, rsqrt_f64(dx * dx + dy_ * dy_ + dz * dz), acc);
+          const double rho = sqrt(y.x * y.x + y.y * y.y + y.z * y.z);
+          const double hx = y.x / rho, hy = y.y / rho, hz = y.z / rho;
+          const double mx = tx - rm * hx, my = ty - rm * hy, mz = tz - rm * hz;
+          const double px = tx - rp * hx, py = ty - rp * hy, pz = tz - rp * hz;
+          const double dm = sqrt(mx * mx + my * my + mz * mz), dp = sqrt(px * px + py * py + pz * pz);
+          acc += shB[s] * (1.0 - (tx * hx + ty * hy + tz * hz)) / (dp * dm * (dp + dm));
+        }
+      } else if (ch.type == 2) {
 #pragma unroll 2
         for (int s = 0; s < cnt; ++s) {
           const dbl4 y = shA[s];
@@ -227,14 +246,15 @@ __global__ __launch_bounds__(kF64Threads) void k_pairs_f64(const SysDev* __restr
 int pairs_f64_occupancy()
 {
   int b = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_pairs_f64, kF64Threads, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_pairs_f64<false>, kF64Threads, 0);
   return b;
 }
 
-void launch_pairs_f64(int grid, const SysDev* sys, PairWork w1, PairWork w2, const dbl4* src64,
+void launch_pairs_f64(bool wide, int grid, const SysDev* sys, PairWork w1, PairWork w2, const dbl4* src64,
                       const dbl4* surf64_a, const double* surf64_b, double* part64, cudaStream_t st, bool pdl)
 {
-  launch_k(k_pairs_f64, grid, kF64Threads, 0, st, pdl, sys, w1, w2, src64, surf64_a, surf64_b, part64);
+  launch_k(wide ? k_pairs_f64<true> : k_pairs_f64<false>, grid, kF64Threads, 0, st, pdl, sys, w1, w2, src64, surf64_a,
+           surf64_b, part64);
 }
 
 }  // namespace hsma

@@ -385,7 +385,7 @@ static int launch_energy(hsma_server_t* s, EnergySlot& sl, int chain)
       SCK(cudaMemsetAsync(sl.ctr_d, 0, sizeof(unsigned int), sl.st));
       const hsma::PairWork w1{sl.items_d + beg, cnt, sl.ctr_d, std::min(grid * nw, cnt)}, none{nullptr, 0, nullptr, 0};
       if (e->prec == HSMA_FP64)
-        hsma::launch_pairs_f64(grid, e->sys_d, w1, none, e->src64_d, e->surf64a_d, e->surf64b_d, e->part64_d, sl.st);
+        hsma::launch_pairs_f64(e->wide_shells(), grid, e->sys_d, w1, none, e->src64_d, e->surf64a_d, e->surf64b_d, e->part64_d, sl.st);
       else
         hsma::launch_pairs_f32(e->L.cfg, grid, e->sys_d, w1, none, e->srchi_d, e->srclo_d, e->surfa_d, e->surfb_d,
                                e->boxes_d, e->part_d, sl.st);

@@ -211,3 +211,31 @@ def test_fp64_reciprocal_roots():
     fast = (d2 >= np.ldexp(np.longdouble(1.0), -959)) & (d2 < np.ldexp(np.longdouble(1.0), 898))
     assert 0 < fast.sum() < fast.size
     assert (err <= np.where(fast, 2.0 ** -53 + 2.0 ** -58, 2.0 ** -52)).all(), err.max() * 2.0 ** 53
+
+
+@pytest.mark.parametrize("tau, dy_rel", [(0.1, 0.4), (0.01, 0.08), (0.25, 0.1)])
+def test_fp64_dipole_shells_among_the_charges(tau, dy_rel):
+    """The FP64 path's central difference with its inner shell inside the cavity, where charges come
+    close to it (here within d = 1e-6 a, and within 1e-9 a for one), and with the shell outside:
+    against the oracle.  A distance d of points at |x| ~ a is known to 2^-52 a / d on either side;
+    a few such roundings of the nearest point's term, which is the largest, are allowed."""
+    rng = np.random.default_rng(190860)
+    P = oracle.make_params(a=1.0, eps1=2.0, eps2=80.0, kappa=1.5, p=12, M=200, tau=tau, dy_rel=dy_rel)
+    F2 = 99
+    F1, j = round(F2 * (5.0 ** 0.5 - 1.0) / 2.0), np.arange(3, 97, 6)
+    z = -1.0 + 2.0 * j / F2
+    c, ang = z + np.sin(np.pi * z) / np.pi, np.pi * j * F1 / F2
+    yhat = np.stack([np.sqrt(1.0 - c * c) * np.cos(ang), np.sqrt(1.0 - c * c) * np.sin(ang), c], 1)
+    r = min((1.0 + tau) * (1.0 - 0.5 * dy_rel), 0.99)
+    d = np.where(j == 3, 1e-9, 1e-6)
+    xyz = np.concatenate([yhat * (r - d)[:, None], inputs.uniform_ball(rng, 100, 0.7)])
+    q = rng.choice([-1.0, 1.0], len(xyz))
+    h = api.hsma_create(1.0, 2.0, 80.0, 1.5, api.hsma_default_params(p=12, M=200, tau=tau, dy_rel=dy_rel,
+                                                                     precision=api.HSMA_FP64))
+    api.hsma_build_sources(h, xyz, q)
+    err = np.abs(api.hsma_potential(h, api.HSMA_REACTION) - oracle.hsma(P, xyz, q)["phi_rf"])
+    ref = np.abs(oracle.hsma(P, xyz, q)["phi_rf"])
+    near = np.concatenate([d, np.full(100, 1e-2)])
+    if r == 0.99:
+        near[:] = 1e-2
+    assert (err <= 16 * 2.0 ** -52 / near * ref + 1e-12 * np.linalg.norm(ref[-100:])).all()
