@@ -552,7 +552,9 @@ __global__ __launch_bounds__(256) void k_move_charge(const SysDev* __restrict__ 
     }
   }
   __syncthreads();
-  const double rn = sqrt(R.x * R.x + R.y * R.y + R.z * R.z), ro = sqrt(xo * xo + yo * yo + zo * zo);
+  // (separately rounded, as the image's own radius)
+  const double rn = sqrt(__dadd_rn(__dadd_rn(__dmul_rn(R.x, R.x), __dmul_rn(R.y, R.y)), __dmul_rn(R.z, R.z)));
+  const double ro = sqrt(xo * xo + yo * yo + zo * zo);
   const double cn = S.dbar * (S.Rt_a * (rn * S.inv_a) - 1.0) * 0.5;
   const double co = S.dbar * (S.Rt_a * (ro * S.inv_a) - 1.0) * 0.5;
   for (int idx = threadIdx.x; idx < P; idx += blockDim.x) {
@@ -580,15 +582,14 @@ __global__ __launch_bounds__(256) void k_move_charge(const SysDev* __restrict__ 
       float hx, hy, hz, lx, ly, lz;
       // (the lo records' fourth components: the weights of the symmetric pair sum's transposed
       // Kelvin term, as written by k_images)
-      const double rn2 = rn;
       split_hilo(R.x, hx, lx); split_hilo(R.y, hy, ly); split_hilo(R.z, hz, lz);
       src_hi[sr] = make_float4(hx, hy, hz, (float)(S.kc * qk));
-      src_lo[sr] = make_float4(lx, ly, lz, In.centre ? 0.f : (float)(In.Q * rn2));
+      src_lo[sr] = make_float4(lx, ly, lz, In.centre ? 0.f : (float)(In.Q * rn));
       const long long b = S.bb + ks / kBox, bk = b + (S.n + kBox - 1) / kBox;
       box_grow(boxes + 2 * b, hx, hy, hz);
       split_hilo(In.x, hx, lx); split_hilo(In.y, hy, ly); split_hilo(In.z, hz, lz);
       src_hi[sk] = make_float4(hx, hy, hz, (float)In.Q);
-      src_lo[sk] = make_float4(lx, ly, lz, In.centre ? (float)(1e15 * S.inv_a) : (float)(1.0 / rn2));
+      src_lo[sk] = make_float4(lx, ly, lz, In.centre ? (float)(1e15 * S.inv_a) : (float)(1.0 / rn));
       if (!In.centre) box_grow(boxes + 2 * bk, hx, hy, hz);
     }
   }
