@@ -665,7 +665,9 @@ __device__ __forceinline__ float m2p(const float4* M, float4 gc, float4 th, floa
   const float ir = inv_unit(gc.w);
   const float ux = ((th.x - gc.x) + tl.x) * ir, uy = ((th.y - gc.y) + tl.y) * ir, uz = ((th.z - gc.z) + tl.z) * ir;
   const float r2 = ux * ux + uy * uy + uz * uz;
-  const float i2 = __fdividef(1.f, r2), ri = rsqrt_mufu(r2);
+  float i2 = __fdividef(1.f, r2);
+  i2 = fmaf(i2, fmaf(-r2, i2, 1.f), i2);  // (a Newton step: 1/r2 to its rounding, as a division)
+  const float ri = rsqrt_mufu(r2);
   const float px = ux * i2, py = uy * i2, wz = uz * i2;
   float sr = 0.f, si = 0.f;
   // groups of column pairs, the highest first
