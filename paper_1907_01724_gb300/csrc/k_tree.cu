@@ -96,20 +96,11 @@ __device__ __forceinline__ float warp_max(float v)
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
-__device__ __forceinline__ float warp_sum(float v)
+// Sums of 32 values over the warp's lanes, transposed: lane l returns the sum of value l, added
+// pairwise in the order of a butterfly (lanes 16 apart first, then 8, 4, 2, 1).  31 shuffles, where a
+// butterfly for each value takes 160.
+__device__ __forceinline__ float warp_sums(float (&v)[32], int lane)
 {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Sums of N <= 32 values over the warp's lanes, transposed: lane l returns the sum of value l
-// (garbage for l >= N).  31 shuffles for 32 sums, where a butterfly for each takes 160; the same
-// pairs are added, so the sums are those of warp_sum to the bit.
-template <int N>
-__device__ __forceinline__ float warp_sums(float (&v)[N], int lane)
-{
-  static_assert(N == 32, "one value per lane");
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const bool up = lane & o;
