@@ -1624,6 +1624,8 @@ const Engine::Tuned* Engine::tuned_entry(const std::vector<int64_t>& ns) const
 // cavity on a GB300, in us, for K = 1, 2 and 4 (128, 64 and 64 threads; 4, 4 and 8 items per slot):
 //   N = 700 (W = 1.9e6) 33.0, 35.6, 43.4; N = 2000 (1.1e7) 39.2, 41.5, 53.6;
 //   4 x 2000 (4.2e7) 59.5, 53.1, 58.5; N = 4999 (5.6e7) 66.5, 57.7, 61.8;
+//   K = 2 and 4: N = 5500 (6.8e7) 60.1, 64.8; 64 x 500 (7.4e7) 160.4, 176.8; N = 6000 (8.0e7) 73.5,
+//   65.7; N = 7000 (1.07e8) 74.2, 70.0; 16 x 1600 (1.15e8) 127.4, 123.9;
 //   N = 10000 (2.3e8) 154, 114, 107.6; 16 x 3000 (3.3e8) 270, 221, 205.5;
 //   N = 40000 (3.3e9) 1445, 903, 718.
 // (At N = 2000 the smallest groups would save 2 us a step, but their 63 x 64 items cost a first pass
@@ -1637,7 +1639,7 @@ int Engine::choose_config(const std::vector<int64_t>& ns) const
   for (size_t s = 0; s < ns.size(); ++s) W += (double)ns[s] * (2.0 * (double)ns[s] + 1.3 * spec[s].M);
   if (const Tuned* e = tuned_entry(ns)) return e->cfg;
   static const int small = config_of(128, 1, 4), medium = config_of(64, 2, 4), large = config_of(64, 4, 8);
-  return W < 6.0e6 ? small : (W < 1.2e8 ? medium : large);
+  return W < 6.0e6 ? small : (W < 7.5e7 ? medium : large);
 }
 
 // Tile configuration of the field pass: a forced or autotuned one is the pair pass's; else by the same

@@ -144,10 +144,10 @@ def _with_tiles(s, tiles, evaluate):
     return evaluate(b)
 
 
-TILES = [(128, 1, 4), (64, 2, 4), (64, 4, 8)]  # by work: below 6e6, below 1.2e8, above
+TILES = [(128, 1, 4), (64, 2, 4), (64, 4, 8)]  # by work: below 6e6, below 7.5e7, above
 
 
-@pytest.mark.parametrize("line, n", [(6.0e6, 1437), (1.2e8, 7427)])
+@pytest.mark.parametrize("line, n", [(6.0e6, 1437), (7.5e7, 5807)])
 def test_tile_rule_on_both_sides_of_its_lines(line, n):
     """The untuned choice by the work N (2 N + 1.3 M), M = 1000, for the last size below a line and the
     first above it: the potentials are those of that configuration to the bit, not those of the
