@@ -1643,17 +1643,18 @@ int Engine::choose_config(const std::vector<int64_t>& ns) const
 }
 
 // Tile configuration of the field pass: a forced or autotuned one is the pair pass's; else by the same
-// work W the pair pass's smallest groups, and from there CTAs of 128 threads with 4 targets each.  The
-// pair pass's own choices serve the field worse: a chunk costs every target 32 bytes of partials, and
-// CTAs of 64 threads stage each source for half as many targets.  Field steps with the pair pass's
-// tiles and with these, in us, passes on several streams: N = 5000 68.1 and 61.5, 9000 145.2 and 142.7,
-// 13001 262 and 251, 16000 361 and 339, 20000 527 and 519, 40000 1772 and 1750; 64 x 1000 375 and 367.
-// (Alone on the GPU, where longer items end less evenly, the first are faster at some sizes: N = 9000
-// 170 and 178, 20000 586 and 606, 30000 1175 and 1192, but 13001 290 and 287, 16000 431 and 418.)
+// work W the pair pass's smallest groups, and from there CTAs of 64 threads with 4 targets each and half
+// as many items as the pair pass takes for its largest sizes: a chunk costs every target 32 bytes of
+// partials.  Field steps with the pair pass's tiles and with these, in us, passes on several streams:
+// N = 5000 68.1 and 60.5, 9000 145.2 and 143.9, 13001 262 and 250, 16000 361 and 340, 20000 527 and 520,
+// 40000 1772 and 1768; 64 x 1000 375 and 368.  (Alone on the GPU the first are faster at some sizes,
+// N = 9000 170 and 178, 20000 586 and 605, 30000 1175 and 1183, and slower at others, 13001 290 and 285,
+// 16000 431 and 416.)  CTAs of 128 threads are as fast, but sum 128 sources in FP32 before a fold, not
+// 64: over 27 cavities their errors are 1.12 (fields) and 1.46 (potentials) times these.
 int Engine::choose_field_config(const std::vector<int64_t>& ns) const
 {
   const int cfg = choose_config(ns);
-  static const int small = config_of(128, 1, 4), field = config_of(128, 4, 4);
+  static const int small = config_of(128, 1, 4), field = config_of(64, 4, 4);
   return forced_cfg >= 0 || tuned_entry(ns) || cfg == small ? cfg : field;
 }
 

@@ -166,11 +166,11 @@ def test_tile_rule_on_both_sides_of_its_lines(line, n):
         assert np.linalg.norm(phi - ref) <= 1e-6 * np.linalg.norm(ref)
 
 
-@pytest.mark.parametrize("n, tiles", [(300, (128, 1, 4)), (1437, (128, 1, 4)), (1438, (128, 4, 4)), (7428, (128, 4, 4)),
-                                      (20000, (128, 4, 4))])
+@pytest.mark.parametrize("n, tiles", [(300, (128, 1, 4)), (1437, (128, 1, 4)), (1438, (64, 4, 4)), (7428, (64, 4, 4)),
+                                      (20000, (64, 4, 4))])
 def test_field_pass_has_its_own_tiles(n, tiles):
     """The untuned field pass, M = 1000: the pair pass's smallest tiles below a work N (2 N + 1.3 M) of
-    6e6, CTAs of 128 threads with 4 targets each above, whatever the pair pass takes there: fields and
+    6e6, CTAs of 64 threads with 4 targets each above, whatever the pair pass takes there: fields and
     the potentials of the same pass are those of that configuration to the bit, potentials of a later
     pass again those of the pair pass, and the chunks cover every source (1e-6 of the FP64 field pass)."""
     rng = np.random.default_rng(190890 + n)
