@@ -454,8 +454,8 @@ __global__ __launch_bounds__(kF64FThreads) void k_field_f64(const SysDev* __rest
         for (int s = 0; s < cnt; ++s) {
           const dbl4 h = shA[s];
           if (ch.type == 0 && sb + s == i) continue;
-          // separately rounded IEEE operations, as in the potential (a charge next to its own
-          // Kelvin image is an ill-conditioned distance)
+          // separately rounded IEEE operations, a root and divisions (the potential pass takes
+          // rsqrt_f64: the two passes' potentials agree to FP64 rounding, not to the bit)
           const double dx = tg.x - h.x, dy = tg.y - h.y, dz = tg.z - h.z;
           const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
           const double d = sqrt(r2);

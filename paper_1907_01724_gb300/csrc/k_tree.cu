@@ -11,10 +11,11 @@
 // which form one expansion about the centre instead.
 //   k_tree_marks  record range of every node of levels kTreeTop..L (first and last position of
 //                 each key prefix)
-//   k_tree_leaf   level L: bounding box, centre, radius and the multipole moments of both trees
-//                 (a warp per node, lane-strided records, fixed-order warp sums)
+//   k_tree_leaf   level L: bounding box, centre, radius and the multipole moments (a warp per node
+//                 and tree, lane-strided records, fixed-order warp sums)
 //   k_tree_up     levels L-1..kTreeTop: box and radius from the children, moments by shifting
-//                 the children's moments to the parent's centre (a warp per node)
+//                 the children's moments to the parent's centre (a block per node and tree, a warp
+//                 per child, or per two children at order 16)
 //   k_tree_far    the far images' expansion about the centre (fixed-order block sums, the last
 //                 block adds the blocks in order)
 //   k_tree_eval   persistent warps over items (32 consecutive targets, one tree, an eighth of
@@ -22,8 +23,9 @@
 //                 level-kTreeTop cells; a node far from every target of the group (radius <=
 //                 theta (distance of the target from the centre)) with at
 //                 least cmin records is evaluated from its moments at each target, a near leaf (or a
-//                 far node too small for its moments to pay) by the direct pair sum with hi/lo
-//                 coordinate differences; then the far-image expansion at each target.  Writes the
+//                 far node too small for its moments to pay) by the direct pair sum, with FP32
+//                 coordinates relative to the node's centre or, next to it, hi/lo differences
+//                 (p2p); then the far-image expansion at each target.  Writes the
 //                 real and the Kelvin sums as the (hi, lo) partials of chunks 0..kTreeRootSplit-1
 //                 and kTreeRootSplit..2 kTreeRootSplit-1, which the reduction adds as it adds every
 //                 chunk.
@@ -712,11 +714,15 @@ __device__ __forceinline__ float l2p_far(const float2* __restrict__ L, float4 th
 //    distance, e.g. a charge next to its own Kelvin image); checked: the node holds some of the
 //    group's own targets, and the source at sorted position `self` is skipped.
 //  Otherwise, for a node whose radius is at most kRelRadius times its distance from every target:
-//    the difference of the FP32 coordinates relative to the node's centre c.  With
-//    X = |t - c| + rho and d >= |t - c| - rho the rounding of either is at most sqrt(3) u X / d
-//    relative to the distance (u = 2^-24), X / d <= 4: 8e-7, and of either sign.  9 operations for
-//    two pairs instead of 15, half the shared loads and half the staging; nine tenths of the direct pairs
-//    at N = 1e5.
+//    the difference of the FP32 coordinates relative to the node's centre c.  Two roundings form a
+//    coordinate (its hi part less the centre's, which is mostly exact, and the lo part), one the
+//    difference; with d >= |t - c| - rho the distance d is off by at most u (1 + 2 (1 + r)/(1 - r)) = 9 u
+//    = 5.4e-7 of it (u = 2^-24, r = kRelRadius), of either sign.  9 operations for two pairs instead of
+//    15, half the shared loads and half the staging; nine tenths of the direct pairs at N = 1e5 (step
+//    2.27 ms, 2.66 with hi/lo differences throughout; 23.4 and 24.5 at N = 1e6).  Over 40 drawn cavities
+//    (N = 20000 to 200000, theta 0.4 to 0.6, orders 8, 12 and 16) the potentials' errors against the FP64
+//    path are 1.0008 times those with hi/lo differences throughout, and 0.866 times those before the
+//    series by column pairs.
 // kelvin: records beyond rfar2 count as zero.  Each batch's FP32 sum is added to the compensated
 // total (a leaf of a dense cluster holds thousands of sources of similar size and mixed sign).
 constexpr float kRelRadius = 0.6f;
@@ -859,8 +865,8 @@ __device__ __forceinline__ void eval_group(const TreeView& t, float2* __restrict
       const bool far = rm * rm <= theta2 * d2;
       if (far && be.y - be.x >= t.cmin) {
         // the order whose truncation at the group's largest ratio rho/|t - c| stays within a tenth
-        // of the order-P bound at theta: (q + 1) log(ratio) <= log(0.1 theta^(P+1)); order 16 keeps
-        // every node at its order
+        // of the order-P bound at theta: (q + 1) log(ratio) <= log(0.1 theta^(P+1)) (the divisions'
+        // last bits move an order only next to a whole number); order 16 keeps every node at its order
         int q = P;
         if constexpr (P <= 12) {
           q = min(P, max(2, (int)ceilf(__fdividef(t.log_eps, 0.5f * __logf(__fdividef(rm * rm, d2)))) - 1));

@@ -40,7 +40,7 @@ struct TreeView {
   int2* node;                // [nodes]: record range [begin, end) of every node
   float4* geo;               // [2][nodes]: centre and radius of the real / Kelvin sources (radius < 0: none)
   float4* box;               // [2][nodes][2]: bounding box (min, max) of the same
-  float4* mom;               // [2][nodes][nq]: multipole moments about the centre, in units of the radius
+  float4* mom;               // [2][nodes][nq]: multipole moments about the centre, in units of 1/inv_unit(radius)
   float2* farp;              // [kFarBlocks][tree_nm(kFarOrder)]: block partials of the far-image expansion
   float2* farL;              // [tree_nm(kFarOrder)]: the far-image expansion
   unsigned int* ctr;         // [0]: completion counter of k_tree_far, [1]: k_tree_eval's work counter
