@@ -245,9 +245,8 @@ int hsma_batch_workspace_size(hsma_batch_t* b, const int64_t* n, size_t* bytes)
   std::vector<int64_t> ns(n, n + b->e->spec.size());
   // the largest layout over all tile configurations, so that a workspace of this size also
   // serves the autotuner, and the untuned one (whose field pass may have its own)
-  const bool f64 = b->e->prec == HSMA_FP64;
-  size_t mx = b->e->make_layout(ns, f64 ? 0 : b->e->choose_config(ns), f64 ? 0 : b->e->choose_field_config(ns), true).bytes;
-  for (int c = 0; c < (f64 ? 0 : hsma::pair_config_count()); ++c)
+  size_t mx = b->e->workspace_bytes(ns);
+  for (int c = 0; b->e->prec != HSMA_FP64 && c < hsma::pair_config_count(); ++c)
     mx = std::max(mx, b->e->make_layout(ns, c, c, true).bytes);
   *bytes = mx;
   return HSMA_OK;

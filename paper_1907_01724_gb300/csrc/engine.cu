@@ -437,8 +437,8 @@ Layout Engine::make_layout(const std::vector<int64_t>& ns, int cfg, int fcfg, bo
         d.chunk_s = c.chunk_s;
         d.ncs = c.ncs;
         // the field pass: by its own configuration (choose_field_config)
-        const Chunking f = fcfg == cfg ? c : chunks_f32(n, sp.M, 32 * pair_config(fcfg).k, std::max(1.0, std::round(
-                                                           desired_of(fcfg) * share)));
+        const double items_f = std::max(1.0, std::round(desired_of(fcfg) * share));
+        const Chunking f = fcfg == cfg ? c : chunks_f32(n, sp.M, 32 * pair_config(fcfg).k, items_f);
         d.fchunk = f.chunk;
         d.fncr = f.ncr;
         d.fchunk_s = f.chunk_s;
@@ -799,8 +799,8 @@ int Engine::attach(void* ptr, size_t bytes)
 int Engine::set_sizes(const std::vector<int64_t>& ns)
 {
   if (have_layout && ns == cur_ns && layout_uploaded) return HSMA_OK;
-  const int cfg = prec == HSMA_FP64 ? 0 : choose_config(ns);
-  L = make_layout(ns, cfg, prec == HSMA_FP64 ? 0 : choose_field_config(ns));
+  const int cfg = choose_config(ns);
+  L = make_layout(ns, cfg, choose_field_config(ns));
   rk_side = prec == HSMA_FP64 ? 1 : choose_side(ns);
   cur_ns = ns;
   have_layout = true;
@@ -1634,6 +1634,7 @@ const Engine::Tuned* Engine::tuned_entry(const std::vector<int64_t>& ns) const
 // takes 110.7, 258.8 and 735.5 at N = 10000, 20000 and 40000 against 107.6, 251.1 and 717.8.
 int Engine::choose_config(const std::vector<int64_t>& ns) const
 {
+  if (prec == HSMA_FP64) return 0;
   if (forced_cfg >= 0) return forced_cfg;
   double W = 0.0;
   for (size_t s = 0; s < ns.size(); ++s) W += (double)ns[s] * (2.0 * (double)ns[s] + 1.3 * spec[s].M);
@@ -1653,9 +1654,16 @@ int Engine::choose_config(const std::vector<int64_t>& ns) const
 // 64: over 27 cavities their errors are 1.12 (fields) and 1.46 (potentials) times these.
 int Engine::choose_field_config(const std::vector<int64_t>& ns) const
 {
+  if (prec == HSMA_FP64) return 0;
   const int cfg = choose_config(ns);
   static const int small = config_of(128, 1, 4), field = config_of(64, 4, 4);
   return forced_cfg >= 0 || tuned_entry(ns) || cfg == small ? cfg : field;
+}
+
+// Bytes of the layout that set_sizes makes for these sizes.
+size_t Engine::workspace_bytes(const std::vector<int64_t>& ns) const
+{
+  return make_layout(ns, choose_config(ns), choose_field_config(ns), true).bytes;
 }
 
 // Schedule of the real/Kelvin pair items in the fused graph: forced, else the size class's
@@ -1832,8 +1840,7 @@ const char* hsma_last_error(const hsma_t* h)
 int hsma_workspace_size(hsma_t* h, int64_t n, size_t* bytes)
 {
   if (!h || !bytes || n < 0 || n > (int64_t)INT32_MAX / 4) return set_err(h, HSMA_E_INVALID_ARG, "bad argument");
-  const bool f64 = h->e->prec == HSMA_FP64;
-  *bytes = h->e->make_layout({n}, f64 ? 0 : h->e->choose_config({n}), f64 ? 0 : h->e->choose_field_config({n}), true).bytes;
+  *bytes = h->e->workspace_bytes({n});
   return HSMA_OK;
 }
 

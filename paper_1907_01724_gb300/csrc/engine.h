@@ -110,6 +110,7 @@ class Engine {
   int apply_move(int64_t k, const double* x_new);
   int choose_config(const std::vector<int64_t>& ns) const;
   int choose_field_config(const std::vector<int64_t>& ns) const;
+  size_t workspace_bytes(const std::vector<int64_t>& ns) const;
   int choose_side(const std::vector<int64_t>& ns) const;
   int autotune(int reps, int* best, float* best_ms);
   int tune_time_config(int c, int side, int steps, std::vector<float>& t);  // (autotune) steps after a rebuild

@@ -720,8 +720,7 @@ int hsma_server_load(hsma_server_t* s, const int64_t* n, const double* xyz, cons
     // device footprint of the chain on its own
     Engine& e = *s->e;
     e.spec = {s->specs[c]};
-    const int cfg = e.prec == HSMA_FP64 ? 0 : e.choose_config({n[c]});
-    s->footprint[c] = e.make_layout({n[c]}, cfg, cfg, true).bytes;
+    s->footprint[c] = e.workspace_bytes({n[c]});
     off += n[c];
   }
   int rc = admit(s, admitted);
